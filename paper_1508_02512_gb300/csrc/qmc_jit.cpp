@@ -42,7 +42,7 @@
 
 namespace {
 
-#define QMC_JIT_GENERATOR_VERSION 8u
+#define QMC_JIT_GENERATOR_VERSION 9u
 #define QMC_GEN_INLINE_TERMS 2048 /* families with more terms get out-of-line sector functions */
 
 const PackedHeader *hdr(const void *p) {
@@ -120,30 +120,44 @@ int top_var(Key k, int S) {
 
 /* Spelling of the generated code in one precision */
 struct Lang {
-    bool f64;
-    bool x2;  /* two lattice points per thread, one per lane of the packed FP32 instructions */
-    const char *real, *cplx, *mk, *cmul, *term, *pre, *pol, *body;
+    bool f64; /* else FP32 with two lattice points per thread, one per lane of the packed instructions */
+    const char *real, *cplx, *mk, *term, *pre, *pol, *body;
     const char *zero_r, *zero_c, *cre, *cim; /* zero values and the members of a complex value */
 };
-const Lang kF32{false, true, "float2", "c2", "mkc2", "cmul2", "float4", "qg", "QgPol", "eval_f32x2_body",
+const Lang kF32{false, "float2", "c2", "mkc2", "float4", "qg", "QgPol", "eval_f32x2_body",
                 "bc2(0.f)", "zero_c2()", "re", "im"};
-const Lang kF64{true, false, "double", "cd", "mk", "cmul", "PackedTerm", "qd", "QdPol", "eval_f64_body",
+const Lang kF64{true, "double", "cd", "mk", "PackedTerm", "qd", "QdPol", "eval_f64_body",
                 "0", "mk(0, 0)", "x", "y"};
+
+/* a term of a polynomial: exponents and its index within the sector */
+struct HTerm {
+    uint8_t e[8];
+    int term;
+    bool dead; /* vanishes on the face t_Y = 0 */
+};
 
 struct PolySet {
     int S = 0;
     bool complex_ = false;
     bool hi_only = false; /* FP32: the coefficient's hi part only (see generate) */
+    bool nested = false;  /* in Horner form (emit_horner) instead of a sum over shared monomials */
     int n_acc = 0;
     std::vector<Entry> constants;
     std::map<Key, std::vector<Entry>> mono; /* every needed monomial (terms' and their parents), key -> terms */
+    std::vector<std::vector<HTerm>> by_acc; /* the terms of each polynomial */
 };
 
 /* zeroed: the subset Y of the endpoint subtraction whose coordinates are zero; terms with a positive power of
    one of them vanish there and are left out (adding c * 0 would change nothing) */
 void add_term(PolySet &P, int acc, int term, const uint8_t *e, unsigned zeroed = 0) {
-    for (int j = 0; j < P.S; ++j)
-        if (((zeroed >> j) & 1u) && e[j]) return;
+    HTerm h;
+    std::memcpy(h.e, e, 8);
+    h.term = term;
+    h.dead = false;
+    for (int j = 0; j < P.S; ++j) h.dead = h.dead || (((zeroed >> j) & 1u) && e[j]);
+    P.by_acc.resize(P.n_acc);
+    P.by_acc[acc].push_back(h);
+    if (h.dead) return;
     Key k = key_of(e, P.S);
     if (k == 0) {
         P.constants.push_back({acc, term});
@@ -160,30 +174,20 @@ void add_term(PolySet &P, int acc, int term, const uint8_t *e, unsigned zeroed =
     }
 }
 
-/* one term: FP32 adds (hi + lo) x m with two packed FMAs per component, for both lanes' points (coefficient
-   slot (hi, hi, lo, lo)); FP64 one FMA */
+/* Polynomials as sums over shared monomials: FP32, and the real U~ and F~ in FP64.  One term: in FP32 (hi + lo) x m with
+   two packed FMAs per component, for both lanes' points (coefficient slot (hi, hi, lo, lo)); in FP64 one FMA. */
 void emit_fma(std::string &o, const Lang &L, const PolySet &P, const Entry &E, const std::string &m,
               const std::string &ind) {
     char b[256];
-    if (L.x2) {
+    if (L.f64)
+        std::snprintf(b, sizeof(b), "%sa%d = fma(C[%d].c, %s, a%d);\n", ind.c_str(), E.acc, E.term, m.c_str(), E.acc);
+    else
         std::snprintf(b, sizeof(b), "%sa%d = %s(C[%d], %s, a%d);\n", ind.c_str(), E.acc,
                       P.complex_ ? "cfma2c" : (P.hi_only ? "rfma2h" : "rfma2c"), E.term, m.c_str(), E.acc);
-    } else if (L.f64) {
-        if (!P.complex_)
-            std::snprintf(b, sizeof(b), "%sa%d = fma(C[%d].c, %s, a%d);\n", ind.c_str(), E.acc, E.term, m.c_str(), E.acc);
-        else
-            std::snprintf(b, sizeof(b), "%sa%d.x = fma(C[%d].c, %s.x, a%d.x); a%d.y = fma(C[%d].c, %s.y, a%d.y);\n",
-                          ind.c_str(), E.acc, E.term, m.c_str(), E.acc, E.acc, E.term, m.c_str(), E.acc);
-    } else if (!P.complex_) {
-        std::snprintf(b, sizeof(b), "%sa%d = fmaf(C[%d].hi, %s, fmaf(C[%d].lo, %s, a%d));\n", ind.c_str(), E.acc,
-                      E.term, m.c_str(), E.term, m.c_str(), E.acc);
-    } else {
-        std::snprintf(b, sizeof(b), "%sa%d = cfma2f(C[%d].hi, C[%d].lo, %s, a%d);\n", ind.c_str(), E.acc, E.term,
-                      E.term, m.c_str(), E.acc);
-    }
     o += b;
 }
 
+/* a monomial (its parent times one variable), its terms and its children */
 void emit_node(std::string &o, const Lang &L, const PolySet &P, Key k, const std::string &parent, int depth, int &id) {
     const int j = top_var(k, P.S);
     const std::string ind(4 + 2 * depth, ' ');
@@ -193,12 +197,9 @@ void emit_node(std::string &o, const Lang &L, const PolySet &P, Key k, const std
     o += ind + "{\n";
     if (parent.empty())
         o += ind + "  const " + type + " " + name + " = " + var + ";\n";
-    else if (P.complex_)
-        o += ind + "  const " + type + " " + name + " = " + L.cmul + "(" + parent + ", " + var + ");\n";
-    else if (L.x2)
-        o += ind + "  const " + type + " " + name + " = mul2(" + parent + ", " + var + ");\n";
     else
-        o += ind + "  const " + type + " " + name + " = " + parent + " * " + var + ";\n";
+        o += ind + "  const " + type + " " + name + " = " +
+             (L.f64 ? parent + " * " + var : (P.complex_ ? "cmul2(" : "mul2(") + parent + ", " + var + ")") + ";\n";
     for (const Entry &E : P.mono.at(k)) emit_fma(o, L, P, E, name, ind + "  ");
     for (int jj = j; jj < P.S; ++jj) {
         const Key ch = k + ((Key)1 << (4 * jj));
@@ -208,26 +209,117 @@ void emit_node(std::string &o, const Lang &L, const PolySet &P, Key k, const std
     o += ind + "}\n";
 }
 
+/* Deformed sectors in FP64: every polynomial in nested (multivariate Horner) form, p = r + x_j q with x_j the variable
+   that occurs in most of its terms, q and r treated alike.  On the FP64 pipe (2 lanes per clock and SM, the bound of
+   the FP64 kernels) a nested node costs one FMA (four for complex x_j q), where the sum over shared monomials costs the
+   monomial's product and an FMA per term: per evaluation of the non-planar double box 232 instead of 456 operations for
+   complex U~ and F~, 394 instead of 504 for the gradient and Hessian.  Measured, FP64 pass with 16 shifts: non-planar
+   double box n = 16381 62.1 -> 54.7 ms, massive box n = 262139 6.52 -> 5.69 ms.  The FP32 code keeps the shared monomials: there
+   instruction issue is the bound.  So do the real U~ and F~ of undeformed sectors: with four poles their rounding near
+   the faces is what is left in the sums, and stays as it was (127 operations for the four-pole double box; 73 nested).
+   The nesting is that of all terms on every face t_Y = 0, with the vanishing ones left out: so the code of a face
+   rounds as the full code does where t_Y is negligible, and the two values that the subtraction of Eq. 11 divides by
+   t_j after taking their difference have the same rounding errors there.
+   Code of a node: `a<acc>` of the innermost scope is its value; a coefficient enters where its monomial ends. */
+void emit_horner(std::string &o, const PolySet &P, int acc, std::vector<HTerm> terms, int depth, int &id) {
+    const std::string ind(4 + 2 * depth, ' ');
+    const std::string a = "a" + std::to_string(acc), v = P.complex_ ? "z[" : "t[";
+    bool have = false; /* the accumulator holds a value */
+    for (size_t k = 0; k < terms.size(); ++k) {
+        bool constant = true;
+        for (int j = 0; j < P.S; ++j) constant = constant && terms[k].e[j] == 0;
+        if (!constant) continue;
+        if (terms[k].dead) {
+            terms.erase(terms.begin() + k);
+            break;
+        }
+        const std::string c = "C[" + std::to_string(terms[k].term) + "].c";
+        o += ind + a + (P.complex_ ? ".x" : "") + " = " + c + ";\n";
+        if (P.complex_) o += ind + a + ".y = 0;\n";
+        terms.erase(terms.begin() + k);
+        have = true;
+        break;
+    }
+    while (!terms.empty()) {
+        int best = 0, most = -1;
+        for (int j = 0; j < P.S; ++j) {
+            int n = 0;
+            for (const HTerm &t : terms) n += t.e[j] > 0;
+            if (n > most) {
+                most = n;
+                best = j;
+            }
+        }
+        std::vector<HTerm> q, r;
+        for (HTerm t : terms) {
+            if (t.e[best] > 0) {
+                --t.e[best];
+                q.push_back(t);
+            } else {
+                r.push_back(t);
+            }
+        }
+        terms.swap(r);
+        const std::string x = v + std::to_string(best) + "]";
+        const HTerm *live = nullptr;
+        int n_live = 0;
+        for (const HTerm &t : q)
+            if (!t.dead) {
+                live = &t;
+                ++n_live;
+            }
+        if (n_live == 0) continue;
+        bool leaf = n_live == 1;
+        for (int j = 0; leaf && j < P.S; ++j) leaf = live->e[j] == 0;
+        if (leaf) {
+            const std::string c = "C[" + std::to_string(live->term) + "].c";
+            if (!P.complex_)
+                o += ind + a + (have ? " = fma(" + c + ", " + x + ", " + a + ");\n" : " = " + c + " * " + x + ";\n");
+            else if (have)
+                o += ind + a + ".x = fma(" + c + ", " + x + ".x, " + a + ".x); " + a + ".y = fma(" + c + ", " + x + ".y, " + a +
+                     ".y);\n";
+            else
+                o += ind + a + ".x = " + c + " * " + x + ".x; " + a + ".y = " + c + " * " + x + ".y;\n";
+        } else {
+            const std::string h = "h" + std::to_string(id++);
+            const std::string type = P.complex_ ? "cd" : "double";
+            o += ind + "{\n" + ind + "  " + type + " " + h + ";\n" + ind + "  {\n" + ind + "    " + type + " " + a + ";\n";
+            emit_horner(o, P, acc, q, depth + 2, id);
+            o += ind + "    " + h + " = " + a + ";\n" + ind + "  }\n";
+            if (!P.complex_)
+                o += ind + "  " + a + (have ? " = fma(" + x + ", " + h + ", " + a + ");\n" : " = " + x + " * " + h + ";\n");
+            else if (have)
+                o += ind + "  " + a + ".x = fma(" + x + ".x, " + h + ".x, fma(-" + x + ".y, " + h + ".y, " + a + ".x)); " + a +
+                     ".y = fma(" + x + ".x, " + h + ".y, fma(" + x + ".y, " + h + ".x, " + a + ".y));\n";
+            else
+                o += ind + "  " + a + " = cmul(" + x + ", " + h + ");\n";
+            o += ind + "}\n";
+        }
+        have = true;
+    }
+}
+
 void emit_body(std::string &o, const Lang &L, const PolySet &P) {
     for (int a = 0; a < P.n_acc; ++a)
         o += P.complex_ ? std::string("    ") + L.cplx + " a" + std::to_string(a) + " = " + L.zero_c + ";\n"
                         : std::string("    ") + L.real + " a" + std::to_string(a) + " = " + L.zero_r + ";\n";
+    int id = 0;
+    if (P.nested) {
+        for (size_t a = 0; a < P.by_acc.size(); ++a) emit_horner(o, P, (int)a, P.by_acc[a], 0, id);
+        return;
+    }
     for (const Entry &E : P.constants) {
         char b[160];
-        if (L.x2 && P.hi_only)
+        if (L.f64)
+            std::snprintf(b, sizeof(b), "    a%d += C[%d].c;\n", E.acc, E.term);
+        else if (P.hi_only)
             std::snprintf(b, sizeof(b), "    a%d = add2(a%d, bc2(C[%d].x));\n", E.acc, E.acc, E.term);
-        else if (L.x2)
+        else
             std::snprintf(b, sizeof(b), P.complex_ ? "    a%d.re = add2(a%d.re, bc2(C[%d].x + C[%d].z));\n"
                                                    : "    a%d = add2(a%d, bc2(C[%d].x + C[%d].z));\n",
                           E.acc, E.acc, E.term, E.term);
-        else if (L.f64)
-            std::snprintf(b, sizeof(b), P.complex_ ? "    a%d.x += C[%d].c;\n" : "    a%d += C[%d].c;\n", E.acc, E.term);
-        else
-            std::snprintf(b, sizeof(b), P.complex_ ? "    a%d.x += C[%d].hi + C[%d].lo;\n" : "    a%d += C[%d].hi + C[%d].lo;\n",
-                          E.acc, E.term, E.term);
         o += b;
     }
-    int id = 0;
     for (int j = 0; j < P.S; ++j) {
         const Key k = (Key)1 << (4 * j);
         if (P.mono.count(k)) emit_node(o, L, P, k, "", 0, id);
@@ -323,6 +415,7 @@ std::string generate(const PackedHeader *h, const Lang &L) {
                    coefficients enter rounded to FP32 (hi), so the Jacobian matches the deformation applied to FP32
                    rounding, which bounds that path anyway (measured: 5 % faster, FP32 error unchanged) */
                 P.hi_only = !L.f64;
+                P.nested = L.f64;
                 const int bG = p.nU + p.nF, bH = bG + p.nG;
                 for (int j = 0; j < S; ++j)
                     for (int k = bG + p.gstart[j]; k < bG + p.gstart[j + 1]; ++k) add_term(P, j, k, T[k].e, Y);
@@ -339,6 +432,7 @@ std::string generate(const PackedHeader *h, const Lang &L) {
                 PolySet Q;
                 Q.S = S;
                 Q.complex_ = true;
+                Q.nested = L.f64;
                 Q.n_acc = 2;
                 for (int k = 0; k < p.nU; ++k) add_term(Q, 0, k, T[k].e, Y);
                 for (int k = 0; k < p.nF; ++k) add_term(Q, 1, p.nU + k, T[p.nU + k].e, Y);
