@@ -36,25 +36,13 @@ struct cd {
     double x, y;
 };
 DEV cd mk(double x, double y) { return cd{x, y}; }
-DEV cd cadd(cd a, cd b) { return cd{a.x + b.x, a.y + b.y}; }
 DEV cd csub(cd a, cd b) { return cd{a.x - b.x, a.y - b.y}; }
 DEV cd cscale(cd a, double s) { return cd{a.x * s, a.y * s}; }
 DEV cd cmul(cd a, cd b) { return cd{fma(a.x, b.x, -a.y * b.y), fma(a.x, b.y, a.y * b.x)}; }
-DEV cd cinv(cd a) {
-    const double d = __drcp_rn(fma(a.x, a.x, a.y * a.y));
-    return cd{a.x * d, -a.y * d};
-}
-DEV cd cdiv(cd a, cd b) { return cmul(a, cinv(b)); }
-DEV cd cipow(cd z, int e) {
-    cd r = mk(1.0, 0.0);
-    int k = e < 0 ? -e : e;
-    for (int i = 0; i < k; ++i) r = cmul(r, z);
-    return e < 0 ? cinv(r) : r;
-}
 DEV double ipow(double v, int e) {
-    double r = 1.0;
-    int k = e < 0 ? -e : e;
-    for (int i = 0; i < k; ++i) r *= v;
+    if (e == 0) return 1.0;
+    double r = v;
+    for (int i = e < 0 ? -e : e; i > 1; --i) r *= v;
     return e < 0 ? __drcp_rn(r) : r;
 }
 /* ------------------------------------------------------------------ table-driven FP64 log and atan2 */
@@ -89,20 +77,25 @@ DEV void logtab_init() {
 }
 
 DEV double qatan2(double y, double x) {
+    /* magnitudes compare as the integers of their bit patterns (FP64 compares would run on the FP64 pipe) */
     const double a = fabs(x), b = fabs(y);
-    const bool swap = b > a;
+    const long long ba = __double_as_longlong(a), bb = __double_as_longlong(b);
+    const bool swap = bb > ba;
     const double hi = swap ? b : a, lo = swap ? a : b;
-    if (!(hi > 1e-30 && hi < 1e30 && lo <= hi)) return atan2(y, x); /* zero, tiny, huge or not a number */
+    const long long bh = swap ? bb : ba;
+    if (!(bh > __double_as_longlong(1e-30) && bh < __double_as_longlong(1e30)))
+        return atan2(y, x); /* zero, tiny, huge or not a number */
     const int k = min(max(__float2int_rn(128.f * __fdividef((float)lo, (float)hi)), 0), 128);
     const double c = qmc_logtab.grid[k];
     const double d = fma(-c, hi, lo) * __drcp_rn(fma(c, lo, hi));
     const double d2 = d * d;
     double q = fma(d2, -1.0 / 7.0, 1.0 / 5.0);
     q = fma(q, d2, -1.0 / 3.0);
-    double th = qmc_logtab.atan_c[k] + fma(d * d2, q, d);
-    if (swap) th = 0.5 * QMC_PI - th;
-    if (x < 0.0) th = QMC_PI - th;
-    return copysign(th, y);
+    const double th = qmc_logtab.atan_c[k] + fma(d * d2, q, d);
+    /* the octant: th, pi/2 - th (swapped), pi - th (x < 0), pi/2 + th (both) */
+    const bool neg = __double_as_longlong(x) < 0;
+    const double base = swap ? 0.5 * QMC_PI : (neg ? QMC_PI : 0.0);
+    return copysign(base + (swap != neg ? -th : th), y);
 }
 
 DEV double qlog(double x) {
@@ -124,13 +117,8 @@ DEV double qlog(double x) {
     return fma(e, LN2, qmc_logtab.log_c[k]) + fma(e, LN2_LO, p);
 }
 
-/* principal log */
-DEV cd clog_p(cd z) { return cd{0.5 * qlog(fma(z.x, z.x, z.y * z.y)), qatan2(z.y, z.x)}; }
-/* log(F - i0): a negative real F lies at arg -pi */
-DEV cd clog_mi0(cd z) {
-    double arg = (z.y == 0.0) ? (z.x < 0.0 ? -QMC_PI : 0.0) : qatan2(z.y, z.x);
-    return cd{0.5 * qlog(fma(z.x, z.x, z.y * z.y)), arg};
-}
+/* principal log */ /* of U and of the q_j takes its argument from qatan2; log(F - i0) has a negative real F at -pi */
+DEV double arg_mi0(cd z) { return z.y == 0.0 ? (z.x < 0.0 ? -QMC_PI : 0.0) : qatan2(z.y, z.x); }
 
 /* ------------------------------------------------------------------ periodising transform (Eq. 21, order r) */
 /* t = phi_r(x), tm = phi_r(1-x) = 1 - t, w = phi_r'(x); phi_r' = c_r x^r (1-x)^r, c_r = (2r+1)!/(r!)^2 */
@@ -227,66 +215,152 @@ DEV cd poly_c(const PackedTerm *__restrict__ T, int n, const cd *z) {
     return acc;
 }
 
-/* ------------------------------------------------------------------ det(I - i lam A), A real S x S */
+/* ------------------------------------------------------------------ reciprocals, powers and x on the FP64 pipe
+   The FP64 kernels are bound by the FP64 pipe alone (2 lanes per clock and SM: one warp instruction takes 16 cycles
+   of it, in which the SM can issue 64 others).  It also executes FP64 compares and integer conversions, so the code
+   below compares bit patterns, keeps small integers as doubles, and counts operations rather than instructions. */
+DEV double rcp_seed(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+/* 1/x from an approximation r good to some 20 bits, by one step of Householder's third-order iteration: with
+   e = 1 - x r, 1/x = r (1 + e + e^2 + ...) and the first term left out is e^3 < 2^-57.  Three FMAs; the correctly
+   rounded __drcp_rn takes as much of the FP64 pipe as 5.3 of them (measured), and is left for arguments whose
+   reciprocal could leave the normal range. */
+DEV double qrcp(double x) {
+    const unsigned be = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu; /* biased exponent */
+    if (be - 24u > 1998u) return __drcp_rn(x);
+    const double r = rcp_seed(x);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+/* v^e for e >= 1, inv^|e| for e < 0, inv = 1/v */
+DEV cd cpow_inv(cd v, cd inv, int e) {
+    const cd b = e < 0 ? inv : v;
+    cd r = b;
+    for (int i = e < 0 ? -e : e; i > 1; --i) r = cmul(r, b);
+    return r;
+}
+/* a > 0 (false for NaN), by the bit pattern */
+DEV bool is_positive(double a) {
+    const long long b = __double_as_longlong(a);
+    return b > 0 && b <= 0x7FF0000000000000LL;
+}
+/* transform for the FP64 kernels: t, tm = 1 - t, and xy = x (1 - x), whose product over the variables gives the
+   weight prod_j phi_r'(x_j) = c_r^S (prod_j xy_j)^r at once (weight64) */
+DEV void transform64(int r, double x, double &t, double &tm, double &xy) {
+    const double y = 1.0 - x;
+    const bool lo = __double2hiint(x) < 0x3FE00000; /* 0 < x < 1/2 */
+    const double p = phi_poly(r, lo ? x : y);
+    const double q = 1.0 - p;
+    t = lo ? p : q;
+    tm = lo ? q : p;
+    xy = x * y;
+}
 template <int S>
-DEV cd det_deform(const double (&A)[S][S], double lam) {
+DEV double weight64(int r, double xy) {
+    double c = 1.0; /* c_r^S, folded at compile time for each r */
+    switch (r) {
+        case 0: return 1.0;
+        case 1:
+#pragma unroll
+            for (int j = 0; j < S; ++j) c *= 6.0;
+            return c * xy;
+        case 2:
+#pragma unroll
+            for (int j = 0; j < S; ++j) c *= 30.0;
+            return c * (xy * xy);
+        default:
+#pragma unroll
+            for (int j = 0; j < S; ++j) c *= 140.0;
+            return c * (xy * xy * xy);
+    }
+}
+
+/* The exponents' eps parts B_j of the staged sector and their reciprocals as doubles (stage_sector fills them):
+   conversions and divisions run on the FP64 pipe, so they are made once per block and sector. */
+struct SectorConst {
+    double B[8], rB[8];
+};
+static __shared__ SectorConst qmc_sec;
+
+/* ------------------------------------------------------------------ det(I - i lam A), A = D + T H
+   A_jk = delta_jk (1 - 2 t_j) g_j + T_j h_jk with T_j = t_j (1 - t_j) and h the symmetric Hessian of F (packed upper
+   triangle): a[j] = A_jj, and the off-diagonal entries are those of a symmetric matrix with row j scaled by T_j.
+   T^{-1/2} A T^{1/2} is symmetric, so I - i lam A is similar to a complex symmetric matrix whose Hermitian part is the
+   identity: every Schur complement keeps a Hermitian part >= 1 and elimination needs no pivoting.  Carried out
+   without the square roots, on s_j = M_jj and Z_jk with M_jk = T_j Z_jk:
+     s_i -= T_i (T_k / s_k) Z_ki^2,   Z_ij -= (T_k / s_k) Z_ki Z_kj,   i, j > k.
+   T_k = 0 (a coordinate of the zeroed subset Y) leaves nothing to eliminate.  The first step's Z are imaginary, so its
+   products are real.  About 290 FP64 operations for S = 6 (fewer with zeroed coordinates) instead of the 600 of a
+   pivoted elimination on the full matrix: with the shorter series and logarithms of point_integrand, the FP64 pass of
+   the non-planar double box (n = 16381, 16 shifts) went from 54.7 to 34.3 ms, the massive box's (n = 262139) from 5.69
+   to 4.92 ms. */
+template <int S>
+DEV cd det_deform(const double (&T)[S], const double (&a)[S], const double *h, double lam, unsigned Y) {
+    auto at = [](int i, int j) { return i * S - i * (i - 1) / 2 + (j - i); }; /* i <= j */
     if constexpr (S == 1) {
-        return mk(1.0, -lam * A[0][0]);
+        return mk(1.0, -lam * a[0]);
     } else if constexpr (S == 2) {
-        const double tr = A[0][0] + A[1][1];
-        const double dt = fma(A[0][0], A[1][1], -A[0][1] * A[1][0]);
-        return mk(fma(-lam * lam, dt, 1.0), -lam * tr);
+        const double e2 = fma(a[0], a[1], -(T[0] * T[1]) * (h[1] * h[1]));
+        return mk(fma(-lam * lam, e2, 1.0), -lam * (a[0] + a[1]));
     } else if constexpr (S == 3) {
         /* det(I + cA) = 1 + c tr A + c^2 E2(A) + c^3 det A with c = -i lam */
-        const double tr = A[0][0] + A[1][1] + A[2][2];
-        const double e2 = fma(A[0][0], A[1][1], -A[0][1] * A[1][0]) + fma(A[0][0], A[2][2], -A[0][2] * A[2][0]) +
-                          fma(A[1][1], A[2][2], -A[1][2] * A[2][1]);
-        const double dt = A[0][0] * fma(A[1][1], A[2][2], -A[1][2] * A[2][1]) -
-                          A[0][1] * fma(A[1][0], A[2][2], -A[1][2] * A[2][0]) +
-                          A[0][2] * fma(A[1][0], A[2][1], -A[1][1] * A[2][0]);
+        const double h01 = h[at(0, 1)], h02 = h[at(0, 2)], h12 = h[at(1, 2)];
+        const double t01 = T[0] * T[1], p01 = t01 * (h01 * h01), p02 = T[0] * T[2] * (h02 * h02);
+        const double p12 = T[1] * T[2] * (h12 * h12);
+        const double m01 = fma(a[0], a[1], -p01);
+        const double e2 = fma(a[0], a[2], -p02) + fma(a[1], a[2], -p12) + m01;
+        const double x3 = t01 * T[2] * (h01 * h02 * h12);
+        const double dt = fma(m01, a[2], fma(-a[0], p12, fma(-a[1], p02, x3 + x3)));
         const double l2 = lam * lam;
-        return mk(fma(-l2, e2, 1.0), fma(l2 * lam, dt, -lam * tr));
+        return mk(fma(-l2, e2, 1.0), lam * fma(l2, dt, -(a[0] + a[1] + a[2])));
     } else {
-        /* Gaussian elimination with partial pivoting on J = I - i lam A */
-        cd J[S][S];
+        cd s[S], Z[S * (S + 1) / 2];
 #pragma unroll
-        for (int r = 0; r < S; ++r)
+        for (int j = 0; j < S; ++j) s[j] = mk(1.0, -lam * a[j]);
 #pragma unroll
-            for (int c = 0; c < S; ++c) J[r][c] = mk(r == c ? 1.0 : 0.0, -lam * A[r][c]);
-        cd det = mk(1.0, 0.0);
+        for (int i = 1; i < S; ++i)
 #pragma unroll
-        for (int c = 0; c < S; ++c) {
-            int p = c;
-            double best = fabs(J[c][c].x) + fabs(J[c][c].y);
+            for (int j = i + 1; j < S; ++j) Z[at(i, j)] = mk(0.0, -lam * h[at(i, j)]);
+        cd det = s[0];
+        if (!(Y & 1u)) {
+            /* Z_0i Z_0j = -lam^2 h_0i h_0j; rho = lam^2 T_0 / s_0 with Re s_0 = 1 */
+            const double f = (lam * lam) * T[0] * qrcp(fma(s[0].y, s[0].y, 1.0));
+            const cd rho = mk(f, -s[0].y * f);
 #pragma unroll
-            for (int r = c + 1; r < S; ++r) {
-                const double v = fabs(J[r][c].x) + fabs(J[r][c].y);
-                if (v > best) {
-                    best = v;
-                    p = r;
+            for (int i = 1; i < S; ++i) {
+                const double q = T[i] * (h[at(0, i)] * h[at(0, i)]);
+                s[i].x = fma(rho.x, q, s[i].x);
+                s[i].y = fma(rho.y, q, s[i].y);
+#pragma unroll
+                for (int j = i + 1; j < S; ++j) {
+                    const double hh = h[at(0, i)] * h[at(0, j)];
+                    Z[at(i, j)].x = rho.x * hh;
+                    Z[at(i, j)].y = fma(rho.y, hh, Z[at(i, j)].y);
                 }
             }
-            if (p != c) {
-                det = cscale(det, -1.0);
+        }
 #pragma unroll
-                for (int r = c + 1; r < S; ++r) {
-                    if (r == p) {
+        for (int k = 1; k < S; ++k) {
+            det = cmul(det, s[k]);
+            if (k + 1 < S && !((Y >> k) & 1u)) {
+                const double f = T[k] * qrcp(fma(s[k].x, s[k].x, s[k].y * s[k].y));
+                const cd rho = mk(s[k].x * f, -s[k].y * f);
 #pragma unroll
-                        for (int k = c; k < S; ++k) {
-                            const cd tmp = J[c][k];
-                            J[c][k] = J[r][k];
-                            J[r][k] = tmp;
-                        }
+                for (int i = k + 1; i < S; ++i) {
+                    const cd z = Z[at(k, i)], l = cmul(rho, z), m = cmul(l, z);
+                    s[i].x = fma(-T[i], m.x, s[i].x);
+                    s[i].y = fma(-T[i], m.y, s[i].y);
+#pragma unroll
+                    for (int j = i + 1; j < S; ++j) {
+                        const cd w = Z[at(k, j)];
+                        cd &v = Z[at(i, j)];
+                        v.x = fma(-l.x, w.x, fma(l.y, w.y, v.x));
+                        v.y = fma(-l.x, w.y, fma(-l.y, w.x, v.y));
                     }
                 }
-            }
-            det = cmul(det, J[c][c]);
-            const cd inv = cinv(J[c][c]);
-#pragma unroll
-            for (int r = c + 1; r < S; ++r) {
-                const cd f = cmul(J[r][c], inv);
-#pragma unroll
-                for (int k = c + 1; k < S; ++k) J[r][k] = csub(J[r][k], cmul(f, J[c][k]));
             }
         }
         return det;
@@ -327,122 +401,278 @@ struct TabPol {
 };
 
 /* ------------------------------------------------------------------ sector integrand */
+template <bool B>
+struct EnableIf {};
+template <>
+struct EnableIf<true> {
+    typedef void type;
+};
+
 struct Exps {
     int eU0, eU1, eF0, eF1;
 };
 
-/* G at the point tt (t with the subset Y zeroed): returns its eps^0 value G0 and the eps-coefficient X of
-   its logarithm, so that G(eps) = G0 exp(X eps) (Sec. II, Eq. 9 with the deformation of Eq. 14). */
-template <int S, bool DEF, int MAXM, class Pol>
-DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *tt, const double *ttm, const double *Lt,
-                double lam, int M, const Exps &ex, cd &G0, cd &X, uint32_t &fails) {
-    if constexpr (!DEF) {
-        double U, F;
-        P.UFr(Y, tt, U, F);
-        if (s.kind == 1) F = -F;
-        double g = s.D * ipow(U, ex.eU0) * ipow(F, -ex.eF0);
+/* G at the point tt (t with the subset Y zeroed): returns its eps^0 value G0 and, with needX, the eps-coefficient X of
+   its logarithm, so that G(eps) = G0 exp(X eps) (Sec. II, Eq. 9 with the deformation of Eq. 14).  First the undeformed
+   class, where everything is real. */
+template <int S, class Pol>
+DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *tt, const double *Lt, bool needX,
+                const Exps &ex, double &G0, double &X) {
+    double U, F;
+    P.UFr(Y, tt, U, F);
+    if (s.kind == 1) F = -F;
+    double g = s.D * ipow(U, ex.eU0) * ipow(F, -ex.eF0);
+#pragma unroll
+    for (int j = 0; j < S; ++j)
+        for (int k = 0; k < s.A[j]; ++k) g *= tt[j];
+    G0 = g;
+    X = 0.0;
+    if (needX) {
+        /* eU1 log U - eF1 log F as one logarithm: both are real and positive on this path */
+        double x = qlog(ipow(U, ex.eU1) * ipow(F, -ex.eF1));
 #pragma unroll
         for (int j = 0; j < S; ++j)
-            for (int k = 0; k < s.A[j]; ++k) g *= tt[j];
-        G0 = mk(g, 0.0);
-        X = mk(0.0, 0.0);
-        if (MAXM > 0 && M > 0) {
-            /* eU1 log U - eF1 log F as one logarithm: both are real and positive on this path */
-            double x = qlog(ipow(U, ex.eU1) * ipow(F, -ex.eF1));
-#pragma unroll
-            for (int j = 0; j < S; ++j)
-                if (s.A[j] != -1 && s.B[j] != 0) x = fma((double)s.B[j], Lt[j], x);
-            X = mk(x, 0.0);
-        }
-    } else {
+            if (s.A[j] != -1 && s.B[j] != 0) x = fma(qmc_sec.B[j], Lt[j], x);
+        X = x;
+    }
+}
+
+template <int S, class Pol>
+DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *tt, const double *ttm, const double *Lt,
+                double lam, bool needX, const Exps &ex, cd &G0, cd &X, uint32_t &fails) {
+    double d[S];
+    cd detJ;
+    {
         double g[S], h[S * (S + 1) / 2];
         P.GH(Y, tt, g, h);
-        double A[S][S];
+        double T[S], a[S];
         int p = 0;
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-#pragma unroll
-            for (int k = j; k < S; ++k) {
-                A[j][k] = tt[j] * ttm[j] * h[p];
-                if (k != j) A[k][j] = tt[k] * ttm[k] * h[p];
-                ++p;
-            }
+            T[j] = tt[j] * ttm[j];
+            a[j] = fma(ttm[j] - tt[j], g[j], T[j] * h[p]);
+            d[j] = lam * ttm[j] * g[j];
+            p += S - j;
         }
+        detJ = det_deform<S>(T, a, h, lam, Y);
+    }
+    /* z_j = t_j q_j with q_j = 1 - i d_j */
+    cd z[S];
 #pragma unroll
-        for (int j = 0; j < S; ++j) A[j][j] = fma(ttm[j] - tt[j], g[j], A[j][j]);
-        const cd detJ = det_deform<S>(A, lam);
-        cd z[S], q[S];
+    for (int j = 0; j < S; ++j) z[j] = mk(tt[j], -tt[j] * d[j]);
+    cd U, F;
+    P.UFc(Y, z, ex.eU0 != 0 || needX, U, F);
+    fails += is_positive(F.y) ? 1u : 0u;
+    const double F2 = fma(F.x, F.x, F.y * F.y);
+    cd G = detJ;
+    if (ex.eF0 != 0) {
+        const double f = qrcp(F2);
+        G = cmul(G, cpow_inv(F, mk(F.x * f, -F.y * f), -ex.eF0));
+    }
+    if (ex.eU0 > 0) {
+        G = cmul(G, cpow_inv(U, U, ex.eU0));
+    } else if (ex.eU0 < 0) {
+        const double f = qrcp(fma(U.x, U.x, U.y * U.y));
+        const cd iU = mk(U.x * f, -U.y * f);
+        G = cmul(G, cpow_inv(iU, iU, -ex.eU0));
+    }
+    /* prod_j (t_j q_j)^{A_j}, t_j only for A_j >= 0: a product with q_j is two FMAs, and 1/q_j = (1 + i d_j)/(1 + d_j^2) */
+    double re = s.D, den = 1.0;
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        for (int k = 0; k < s.A[j]; ++k) {
+            re *= tt[j];
+            G = mk(fma(G.y, d[j], G.x), fma(-G.x, d[j], G.y));
+        }
+        for (int k = 0; k > s.A[j]; --k) {
+            den *= fma(d[j], d[j], 1.0);
+            G = mk(fma(-G.y, d[j], G.x), fma(G.x, d[j], G.y));
+        }
+    }
+    if (s.sigma > 0) re *= qrcp(den);
+    G0 = cscale(G, re);
+    X = mk(0.0, 0.0);
+    if (needX) {
+        /* eU1 log U - eF1 log F + sum_j B_j log q_j (and B_j log t_j where A_j != -1).  The moduli of U and of the q_j
+           share one logarithm: U and q_j do not scale with the kinematics, so their powers stay in range. */
+        const double U2 = fma(U.x, U.x, U.y * U.y);
+        double num = 1.0, dnm = 1.0, xr = 0.0;
+        double xi = (double)ex.eU1 * qatan2(U.y, U.x);
+        for (int k = 0; k < ex.eU1; ++k) num *= U2;
+        for (int k = 0; k > ex.eU1; --k) dnm *= U2;
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-            const double d = lam * ttm[j] * g[j];
-            z[j] = mk(tt[j], -tt[j] * d);
-            q[j] = mk(1.0, -d);
-        }
-        const bool needU = ex.eU0 != 0 || (MAXM > 0 && M > 0);
-        cd U, F;
-        P.UFc(Y, z, needU, U, F);
-        fails += (F.y > 0.0) ? 1u : 0u;
-        cd G = cscale(detJ, s.D);
-        if (ex.eU0 != 0) G = cmul(G, cipow(U, ex.eU0));
-        G = cmul(G, cipow(F, -ex.eF0));
-        bool any_mono = false;
-        double mono = 1.0;
-#pragma unroll
-        for (int j = 0; j < S; ++j)
-            for (int k = 0; k < s.A[j]; ++k) {
-                mono *= tt[j];
-                any_mono = true;
+            if (s.B[j] != 0) {
+                if (s.A[j] != -1) xr = fma(qmc_sec.B[j], Lt[j], xr);
+                const double q2 = fma(d[j], d[j], 1.0);
+                for (int k = 0; k < s.B[j]; ++k) num *= q2;
+                for (int k = 0; k > s.B[j]; --k) dnm *= q2;
+                xi = fma(-qmc_sec.B[j], qatan2(d[j], 1.0), xi);
             }
-        if (any_mono) G = cscale(G, mono);
-#pragma unroll
-        for (int j = 0; j < S; ++j)
-            if (s.A[j] != 0) G = cmul(G, cipow(q[j], s.A[j]));
-        G0 = G;
-        X = mk(0.0, 0.0);
-        if (MAXM > 0 && M > 0) {
-            cd x = csub(cscale(clog_p(U), (double)ex.eU1), cscale(clog_mi0(F), (double)ex.eF1));
-#pragma unroll
-            for (int j = 0; j < S; ++j) {
-                if (s.B[j] != 0) {
-                    if (s.A[j] != -1) x.x = fma((double)s.B[j], Lt[j], x.x);
-                    x = cadd(x, cscale(clog_p(q[j]), (double)s.B[j]));
-                }
-            }
-            X = x;
         }
+        const double eF1 = (double)ex.eF1;
+        X.x = fma(0.5, fma(-eF1, qlog(F2), qlog(num * qrcp(dnm))), xr);
+        X.y = fma(-eF1, arg_mi0(F), xi);
     }
 }
 
 /* w(x) * (sector integrand) at x, as series slots 0..M (slot n = coefficient of eps^(n - sigma)).
-   Subtraction of Eq. (11) with alpha = -1, regrouped over the zeroed subsets Y of the singular set S:
-   eps^sigma I = sum_Y G_Y(eps) V_Y(eps),  V_Y = prod_{j in S\Y} eps t_j^{-1+B eps} prod_{j in Y} (1/B_j - eps t_j^{-1+B eps}). */
-template <int S, bool DEF, int MAXM, class Pol>
-DEV void point_integrand(const PackedSector &s, const Pol &P, const double *x, int r, double lam,
-                         const Exps &ex, cd (&out)[MAXM + 1], uint32_t &fails) {
-    double t[S], tm[S], w = 1.0;
+   Subtraction of Eq. (11) with alpha = -1 over the zeroed subsets Y of the singular set: with
+   a_j(eps) = eps t_j^{-1 + B_j eps} = sum_{n >= 1} c_n eps^n, each singular variable turns G into a_j (G - G|_{t_j = 0}) +
+   G|_{t_j = 0} / B_j.  The series a_j are made once per point.  Every variable outside Y brings a factor eps, so G_Y is
+   needed to eps^(M - sigma + |Y|) only: its logarithm X is left out where that is zero, in particular at the point
+   itself (Y empty) whenever the highest order wanted is eps^0. */
+struct Subsets {
+    int sigma, M;
+    unsigned smask;
+    /* highest order of eps to which G_Y is needed, count: the subset's bits in singular-variable numbering */
+    DEV int need(unsigned count) const { return M - sigma + __popc(count); }
+};
+
+/* t, 1 - t, logarithms, weight and the series a_j of a point; false: the weight vanishes there */
+template <int S, int MAXM>
+DEV bool point_setup(const PackedSector &s, const double *x, int r, const Subsets &q, double (&t)[S], double (&tm)[S],
+                     double (&Lt)[S], double (&a)[S][MAXM + 1], double &w) {
     bool bad = false;
 #pragma unroll
     for (int j = 0; j < S; ++j) {
-        double wj;
-        transform(r, x[j], t[j], tm[j], wj);
-        w *= wj;
-        bad |= x[j] == 0.0; /* the weight and t vanish only there: x < 1 after the wrap */
+        double xy;
+        transform64(r, x[j], t[j], tm[j], xy);
+        w = j == 0 ? xy : w * xy;
+        bad |= __double_as_longlong(x[j]) <= 0; /* the weight and t vanish only at x = 0: x < 1 after the wrap */
     }
+    if (bad) return false;
+    w = weight64<S>(r, w);
+    int i = 0;
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        const bool sing = (q.smask >> j) & 1u;
+        Lt[j] = 0.0;
+        if (MAXM > 0 && q.M > 0 && (sing || s.B[j] != 0)) Lt[j] = qlog(t[j]);
+        if (!sing) continue;
+        a[i][0] = qmc_sec.rB[j]; /* the place of eps^0 holds 1/B_j */
+        if (MAXM > 0 && q.M > 0) {
+            double c = __drcp_rn(t[j]);
+            const double bl = qmc_sec.B[j] * Lt[j];
+#pragma unroll
+            for (int n = 1; n <= MAXM; ++n) {
+                if (n > q.M) break;
+                a[i][n] = c;
+                if (n < q.M) c *= bl / n;
+            }
+        }
+        ++i;
+    }
+    return true;
+}
+
+/* V *= eps t^{-1 + B eps} (its variable outside Y) or 1/B - eps t^{-1 + B eps} (inside Y) for a series V that starts at
+   eps^z; a: the variable's series */
+template <int MAXM>
+DEV void subset_factor(double (&V)[MAXM + 1], int z, const double *a, bool inY, int M) {
+#pragma unroll
+    for (int n = MAXM; n >= 0; --n) {
+        if (n > M) continue;
+        double acc = 0.0;
+#pragma unroll
+        for (int k = 0; k <= n; ++k) {
+            if (k < z || (k == n && !inY)) continue;
+            const double f = k == n ? a[0] : (inY ? -a[n - k] : a[n - k]);
+            acc = fma(V[k], f, acc);
+        }
+        V[n] = acc;
+    }
+}
+
+/* Undeformed sectors: sum over Y of G_Y(eps) V_Y(eps), V_Y the product of the variables' factors.  The products over all
+   but the last of the (at most four) variables are made once per point, 2^(sigma - 1) series in local memory.
+   This regrouped sum keeps the rounding of a product of the same factors in the same order for every Y: near the faces
+   t_j = 0 the terms cancel, and what is left there of their rounding is all of the error of a four-pole sector's sum.
+   Bound by the FP64 pipe.  With the series and their products hoisted out of the subset loop, no arithmetic on zero
+   imaginary parts or zero coefficients, and no logarithm where the order does not ask for it, the FP64 passes (16
+   shifts) went from 32.2 to 16.2 ms (four-pole double box, n = 8191) and, with 8 shifts, from 5.36 to 2.88 ms (massless
+   box, n = 65521), with the same point values bit for bit. */
+template <int S, bool DEF, int MAXM, class Pol>
+DEV typename EnableIf<!DEF>::type point_integrand(const PackedSector &s, const Pol &P, const double *x, int r, double,
+                                                  const Exps &ex, cd (&out)[MAXM + 1], uint32_t &) {
 #pragma unroll
     for (int n = 0; n <= MAXM; ++n) out[n] = mk(0.0, 0.0);
-    if (bad) return;
-    const int M = s.M;
-    const unsigned smask = (unsigned)s.sing_mask;
-    double Lt[S];
+    const Subsets q{s.sigma, s.M, (unsigned)s.sing_mask};
+    double t[S], tm[S], Lt[S], a[S][MAXM + 1], w;
+    if (!point_setup<S, MAXM>(s, x, r, q, t, tm, Lt, a, w)) return;
+    constexpr int NPRE = S < 4 ? S : 4; /* variables in the shared products: sigma - 1, at most NPRE - 1 */
+    double pre[1 << (NPRE - 1)][MAXM + 1];
+    const int np = q.sigma < NPRE ? (q.sigma > 0 ? q.sigma - 1 : 0) : NPRE - 1;
 #pragma unroll
-    for (int j = 0; j < S; ++j) Lt[j] = 0.0;
-    if (MAXM > 0 && M > 0) {
+    for (int n = 0; n <= MAXM; ++n) pre[0][n] = n == 0 ? 1.0 : 0.0;
+    for (int i = 0; i < np; ++i)
+        for (int k = 0; k < (1 << i); ++k) {
+            double V[MAXM + 1], W[MAXM + 1];
 #pragma unroll
-        for (int j = 0; j < S; ++j)
-            if (((smask >> j) & 1u) || s.B[j] != 0) Lt[j] = qlog(t[j]);
-    }
-    unsigned Y = 0;
+            for (int n = 0; n <= MAXM; ++n) V[n] = W[n] = pre[k][n];
+            const int z = i - __popc(k);
+            subset_factor<MAXM>(V, z, a[i], false, q.M);
+            subset_factor<MAXM>(W, z, a[i], true, q.M);
+#pragma unroll
+            for (int n = 0; n <= MAXM; ++n) {
+                pre[k][n] = V[n];
+                pre[k + (1 << i)][n] = W[n];
+            }
+        }
+    double o[MAXM + 1];
+#pragma unroll
+    for (int n = 0; n <= MAXM; ++n) o[n] = 0.0;
+    unsigned Y = 0, count = 0;
     do {
+        double tt[S];
+#pragma unroll
+        for (int j = 0; j < S; ++j) tt[j] = (Y >> j) & 1u ? 0.0 : t[j];
+        const int need = q.need(count);
+        double g, X;
+        eval_G<S>(s, P, Y, tt, Lt, MAXM > 0 && need > 0, ex, g, X);
+        double V[MAXM + 1];
+        const unsigned low = count & ((1u << np) - 1u);
+#pragma unroll
+        for (int n = 0; n <= MAXM; ++n) V[n] = pre[low][n];
+        int z = np - __popc(low);
+        for (int i = np; i < q.sigma; ++i) {
+            const bool inY = (count >> i) & 1u;
+            subset_factor<MAXM>(V, z, a[i], inY, q.M);
+            z += inY ? 0 : 1;
+        }
+#pragma unroll
+        for (int n = 0; n <= MAXM; ++n) {
+            if (n > need) break;
+#pragma unroll
+            for (int k = 0; k + n <= MAXM; ++k)
+                if (k >= z && n + k <= q.M) o[n + k] = fma(g, V[k], o[n + k]);
+            if (n < need) {
+                g = g * X;
+                if (n > 0) g *= 1.0 / (n + 1);
+            }
+        }
+        ++count;
+        Y = (Y - q.smask) & q.smask;
+    } while (Y != 0);
+#pragma unroll
+    for (int n = 0; n <= MAXM; ++n) out[n].x = o[n] * w;
+}
+
+/* Deformed sectors (at most two poles in the physical integrals): the subsets are enumerated like a binary counter, and
+   whenever both halves of a bit are done (variable i not zeroed, zeroed) they are combined to
+   a_i (G - G0) + G0 / B_i, so that at most sigma complex series wait, on a stack in local memory. */
+template <int S, bool DEF, int MAXM, class Pol>
+DEV typename EnableIf<DEF>::type point_integrand(const PackedSector &s, const Pol &P, const double *x, int r, double lam,
+                                                 const Exps &ex, cd (&out)[MAXM + 1], uint32_t &fails) {
+#pragma unroll
+    for (int n = 0; n <= MAXM; ++n) out[n] = mk(0.0, 0.0);
+    const Subsets q{s.sigma, s.M, (unsigned)s.sing_mask};
+    double t[S], tm[S], Lt[S], a[S][MAXM + 1], w;
+    if (!point_setup<S, MAXM>(s, x, r, q, t, tm, Lt, a, w)) return;
+    cd st[S][MAXM + 1], cur[MAXM + 1];
+    int sp = 0;
+    unsigned Y = 0, count = 0;
+    for (;;) {
         double tt[S], ttm[S];
 #pragma unroll
         for (int j = 0; j < S; ++j) {
@@ -450,48 +680,45 @@ DEV void point_integrand(const PackedSector &s, const Pol &P, const double *x, i
             tt[j] = zj ? 0.0 : t[j];
             ttm[j] = zj ? 1.0 : tm[j];
         }
-        cd G0, X;
-        eval_G<S, DEF, MAXM>(s, P, Y, tt, ttm, Lt, lam, M, ex, G0, X, fails);
-        double V[MAXM + 1];
-        V[0] = 1.0;
+        const int need = q.need(count);
+        cd X;
+        eval_G<S>(s, P, Y, tt, ttm, Lt, lam, MAXM > 0 && need > 0, ex, cur[0], X, fails);
 #pragma unroll
-        for (int n = 1; n <= MAXM; ++n) V[n] = 0.0;
+        for (int n = 1; n <= MAXM; ++n) {
+            if (n > need) break;
+            cur[n] = cmul(cur[n - 1], X);
+            if (n > 1) cur[n] = cscale(cur[n], 1.0 / n);
+        }
+        int i = 0;
+        for (unsigned b = count; b & 1u; b >>= 1, ++i) {
+            --sp;
+            /* the combined series is needed to this order; its lower half, which a_i raises by one, to one less */
+            const int m = q.M - q.sigma + (i + 1) + __popc(b >> 1);
+            cd d[MAXM + 1];
 #pragma unroll
-        for (int j = 0; j < S; ++j) {
-            if ((smask >> j) & 1u) {
-                const bool inY = (Y >> j) & 1u;
-                const double Bj = (double)s.B[j];
-                double f[MAXM + 1];
-                f[0] = inY ? 1.0 / Bj : 0.0;
-                double c = 1.0 / t[j];
+            for (int n = 0; n < MAXM; ++n) {
+                if (n >= m) break;
+                d[n] = csub(st[sp][n], cur[n]);
+            }
 #pragma unroll
-                for (int n = 1; n <= MAXM; ++n) {
-                    f[n] = inY ? -c : c;
-                    c *= Bj * Lt[j] / n;
-                }
+            for (int n = 0; n <= MAXM; ++n) {
+                if (n > m) break;
+                cd acc = cscale(cur[n], a[i][0]);
 #pragma unroll
-                for (int n = MAXM; n >= 0; --n) {
-                    double acc = 0.0;
-#pragma unroll
-                    for (int k = 0; k <= n; ++k) acc = fma(V[k], f[n - k], acc);
-                    V[n] = acc;
-                }
+                for (int k = 1; k <= n; ++k) acc = mk(fma(a[i][k], d[n - k].x, acc.x), fma(a[i][k], d[n - k].y, acc.y));
+                cur[n] = acc;
             }
         }
-        cd g = G0;
+        ++count;
+        Y = (Y - q.smask) & q.smask;
+        if (Y == 0) break;
 #pragma unroll
-        for (int n = 0; n <= MAXM; ++n) {
-            if (n <= M) {
+        for (int n = 0; n <= MAXM; ++n) st[sp][n] = cur[n];
+        ++sp;
+    }
 #pragma unroll
-                for (int k = 0; k + n <= MAXM; ++k)
-                    if (n + k <= M) out[n + k] = cadd(out[n + k], cscale(g, V[k]));
-                g = cscale(cmul(g, X), 1.0 / (n + 1));
-            }
-        }
-        Y = (Y - smask) & smask;
-    } while (Y != 0);
-#pragma unroll
-    for (int n = 0; n <= MAXM; ++n) out[n] = cscale(out[n], w);
+    for (int n = 0; n <= MAXM; ++n)
+        if (n <= q.M) out[n] = cscale(cur[n], w);
 }
 
 /* ------------------------------------------------------------------ staging a sector into shared memory */
@@ -502,6 +729,11 @@ DEV void stage_sector(const unsigned char *packed, int64_t sectors_off, int64_t 
     int4 *dst = reinterpret_cast<int4 *>(smem);
     constexpr int NS = (int)(sizeof(PackedSector) / 16);
     for (int k = threadIdx.x; k < NS; k += blockDim.x) dst[k] = src[k];
+    if (threadIdx.x < 8) {
+        const double B = (double)ps->B[threadIdx.x];
+        qmc_sec.B[threadIdx.x] = B;
+        qmc_sec.rB[threadIdx.x] = 1.0 / B; /* used for singular variables only: B != 0 there */
+    }
     const int nt = ps->n_terms;
     const int4 *tsrc = reinterpret_cast<const int4 *>(packed + terms_off) + ps->term0;
     int4 *tdst = dst + NS;
