@@ -367,13 +367,18 @@ DEV cd det_deform(const double (&T)[S], const double (&a)[S], const double *h, d
     }
 }
 
+struct Exps {
+    int eU0, eU1, eF0, eF1;
+};
+
 /* ------------------------------------------------------------------ polynomial evaluators (FP64)
    The integrand asks an evaluator for
      UFr(Y, t, U, F)          U~ and F~ at real t (undeformed sectors, Eqs. 7-8),
      GH(Y, t, g, h)           g_j = dF~/dt_j and h_p = d2F~/dt_j dt_k (p over j <= k, row-major upper triangle) at
                               real t, the inputs of the deformation of Eq. 14,
      UFc(Y, z, needU, U, F)   U~ (1 when needU is false) and F~ at the deformed point z,
-   where the coordinates in the subset Y (bit j = variable j) of the endpoint subtraction (Eqs. 10-12) are zero.
+   where the coordinates in the subset Y (bit j = variable j) of the endpoint subtraction (Eqs. 10-12) are zero, and
+     exps(J)               the powers eU0 + eU1 eps and eF0 + eF1 eps of U~ and 1/F~.
    TabPol walks the staged term table (and ignores Y: zero coordinates make those terms vanish); the generated
    FP64 evaluator (run-time compiled per family) holds each sector's monomials, per zeroed subset without the
    terms that vanish there, as straight-line code and reads only the coefficients from the same table. */
@@ -382,6 +387,7 @@ struct TabPol {
     const PackedTerm *T;
     const PackedSector *s;
     DEV static TabPol make(const PackedTerm *T, const PackedSector &s, int) { return TabPol{T, &s}; }
+    DEV static Exps exps(const Job &J) { return Exps{J.eU0, J.eU1, J.eF0, J.eF1}; }
     DEV void UFr(unsigned, const double *t, double &U, double &F) const {
         U = poly_r<S>(T, s->nU, t);
         F = poly_r<S>(T + s->nU, s->nF, t);
@@ -401,6 +407,14 @@ struct TabPol {
 };
 
 /* ------------------------------------------------------------------ sector integrand */
+template <bool B, class T, class F>
+struct Select {
+    typedef F type;
+};
+template <class T, class F>
+struct Select<true, T, F> {
+    typedef T type;
+};
 template <bool B>
 struct EnableIf {};
 template <>
@@ -408,9 +422,6 @@ struct EnableIf<true> {
     typedef void type;
 };
 
-struct Exps {
-    int eU0, eU1, eF0, eF1;
-};
 
 /* G at the point tt (t with the subset Y zeroed): returns its eps^0 value G0 and, with needX, the eps-coefficient X of
    its logarithm, so that G(eps) = G0 exp(X eps) (Sec. II, Eq. 9 with the deformation of Eq. 14).  First the undeformed
@@ -882,7 +893,7 @@ DEV void eval_f64_body(const JobTable &jt) {
             cur = psec;
             cur_job = jb;
         }
-        const Exps ex{J.eU0, J.eU1, J.eF0, J.eF1};
+        const Exps ex = Pol::exps(J);
         const Pol pol = Pol::make(T, sec, psec);
         const uint32_t n = J.n;
         const double invn = J.invn;
@@ -1245,10 +1256,8 @@ DEV float ipowf_(float v, int e) {
     return e < 0 ? __frcp_rn(r) : r;
 }
 DEV cf clogf_p(cf z) { return cf{0.5f * __logf(fmaf(z.x, z.x, z.y * z.y)), atan2f(z.y, z.x)}; }
-DEV cf clogf_mi0(cf z) {
-    const float arg = (z.y == 0.f) ? (z.x < 0.f ? -3.14159265358979f : 0.f) : atan2f(z.y, z.x);
-    return cf{0.5f * __logf(fmaf(z.x, z.x, z.y * z.y)), arg};
-}
+DEV float arg_mi0f(float x, float y) { return (y == 0.f) ? (x < 0.f ? -3.14159265358979f : 0.f) : atan2f(y, x); }
+DEV cf clogf_mi0(cf z) { return cf{0.5f * __logf(fmaf(z.x, z.x, z.y * z.y)), arg_mi0f(z.x, z.y)}; }
 
 DEV float phi_poly_f(int r, float x) {
     switch (r) {
@@ -1359,6 +1368,7 @@ struct TabPolF {
     const PackedTermF *T;
     const PackedSector *s;
     DEV static TabPolF make(const PackedTermF *T, const PackedSector &s, int) { return TabPolF{T, &s}; }
+    DEV static Exps exps(const Job &J) { return Exps{J.eU0, J.eU1, J.eF0, J.eF1}; }
     DEV void UFr(unsigned, const float *t, float &U, float &F) const {
         const SmemTabF tab{T};
         U = poly_rf<S>(tab, 0, s->nU, t);
@@ -1747,7 +1757,7 @@ DEV void eval_f32_body(const JobTable &jt) {
             cur = psec;
             cur_job = jb;
         }
-        const Exps ex{J.eU0, J.eU1, J.eF0, J.eF1};
+        const Exps ex = Pol::exps(J);
         const Pol pol = Pol::make(T, sec, psec);
         const uint32_t n = J.n;
         const float invnf = 1.f / (float)n;
@@ -1841,8 +1851,7 @@ __global__ void __launch_bounds__(256) qmc_eval_kernel_f32(const __grid_constant
  * issued once for both points, the staged coefficients are read once for both, and the control flow of the
  * subtraction subsets is shared.  Each lane rounds exactly as the scalar code of the one-point path does, so a
  * lane's value equals that path's value for its point.  Steps without a packed form run per lane with the scalar
- * code: the transcendentals, the reciprocals and the elimination of the deformation determinant (which would
- * need twice the registers in packed form).
+ * code: the transcendentals and the reciprocals.
  * Coefficients are staged as (hi, hi, lo, lo): one 128-bit shared load gives both packed operands of a term. */
 DEV float2 bc2(float v) { return make_float2(v, v); }
 DEV float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
@@ -1874,26 +1883,11 @@ DEV float2 rfma2h(const float4 &c, float2 m, float2 a) { return fma2(make_float2
 DEV float2 rfma2c(const float4 &c, float2 m, float2 a) {
     return fma2(make_float2(c.x, c.y), m, fma2(make_float2(c.z, c.w), m, a));
 }
-DEV cf lane_c(c2 v, int k) { return cf{lane(v.re, k), lane(v.im, k)}; }
-DEV c2 join_c(cf a, cf b) { return c2{make_float2(a.x, b.x), make_float2(a.y, b.y)}; }
 DEV c2 cinv2(c2 a) {
     const float2 d2 = fma2(a.re, a.re, mul2(a.im, a.im));
     const float2 d = make_float2(__fdividef(1.f, d2.x), __fdividef(1.f, d2.y));
     return c2{mul2(a.re, d), neg2(mul2(a.im, d))};
 }
-DEV c2 cipow2(c2 z, int e) {
-    c2 r = c2{bc2(1.f), bc2(0.f)};
-    int k = e < 0 ? -e : e;
-    for (int i = 0; i < k; ++i) r = cmul2(r, z);
-    return e < 0 ? cinv2(r) : r;
-}
-DEV float2 ipow2(float2 v, int e) {
-    float2 r = bc2(1.f);
-    int k = e < 0 ? -e : e;
-    for (int i = 0; i < k; ++i) r = mul2(r, v);
-    return e < 0 ? make_float2(__frcp_rn(r.x), __frcp_rn(r.y)) : r;
-}
-
 /* the periodising transform of both points (transform_f per lane) */
 DEV void transform2(int r, float2 x, float2 y, float2 &t, float2 &tm, float2 &w) {
     const bool la = x.x <= y.x, lb = x.y <= y.y;
@@ -1920,158 +1914,311 @@ DEV void transform2(int r, float2 x, float2 y, float2 &t, float2 &tm, float2 &w)
     }
 }
 
-/* G at the points tt of both lanes (eval_G_f per lane): its eps^0 value G0 and the eps-coefficient X of its
-   logarithm.  live: lanes whose point is evaluated (a sign failure is counted only there). */
-template <int S, bool DEF, int MAXM, class Pol>
-DEV void eval_G_f2(const PackedSector &s, const Pol &P, unsigned Y, const float2 *tt, const float2 *ttm,
-                   const float2 *Lt, float lam, int M, const Exps &ex, const bool (&live)[2], c2 &G0, c2 &X,
-                   uint32_t &fails) {
-    const float2 D = bc2(s.Df);
-    if constexpr (!DEF) {
-        float2 U, F;
-        P.UFr(Y, tt, U, F);
-        if (s.kind == 1) F = neg2(F);
-        float2 g = mul2(mul2(D, ipow2(U, ex.eU0)), ipow2(F, -ex.eF0));
+/* What the two-point kernels read of the staged sector's exponents at every point (stage_sector_f2 fills it): B_j and
+   1/B_j as floats, and bit sets over the variables, tested where the exponents themselves would be loaded, compared and
+   looped over. */
+struct SectorConstF {
+    float B[8], rB[8];
+    unsigned a1, a2, more; /* A_j >= 1; A_j >= 2; A_j >= 3 */
+    unsigned a, b, l;      /* A_j != 0; B_j != 0; B_j != 0 and A_j != -1 */
+    float one;             /* 1 (see det_sym_f2) */
+};
+static __shared__ SectorConstF qmc_secf;
+
+/* v^e, e known at compile time in the generated kernels */
+DEV float2 rpow2(float2 v, int e) {
+    float2 r = v;
+    for (int i = e < 0 ? -e : e; i > 1; --i) r = mul2(r, v);
+    return e < 0 ? make_float2(__frcp_rn(r.x), __frcp_rn(r.y)) : r;
+}
+DEV c2 cpow2(c2 z, int e) {
+    c2 r = z;
+    for (int i = e < 0 ? -e : e; i > 1; --i) r = cmul2(r, z);
+    return e < 0 ? cinv2(r) : r;
+}
+/* v prod_j tt_j^{A_j} over A_j > 0 */
+template <int S>
+DEV float2 mono2(const PackedSector &s, float2 v, const float2 *tt) {
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        if ((qmc_secf.a1 >> j) & 1u) v = mul2(v, tt[j]);
+        if ((qmc_secf.a2 >> j) & 1u) v = mul2(v, tt[j]);
+        if ((qmc_secf.more >> j) & 1u)
+            for (int k = 2; k < s.A[j]; ++k) v = mul2(v, tt[j]);
+    }
+    return v;
+}
+
+/* det(I - i lam A) at both lanes' points for S >= 4: det_sym_f per lane, in packed arithmetic over the lanes.  n: the
+   imaginary parts -lam b_jk of the symmetric matrix (packed upper triangle), whose real part is the identity: the
+   first elimination step works on imaginary numbers only and keeps 15 complex entries (S = 6) alive instead of 21.
+   Bound by issue and the FP32 pipe: 330 packed instructions for both points; per lane it took 330 twice, and as many
+   moves to swap real and imaginary parts.
+   Signs are folded into the factors, so that each difference is one packed addition (negation is exact).  Where a product
+   is rounded before it is added, the addition is an FMA with a factor 1 that the compiler does not know (it would fuse
+   the packed product into a packed addition). */
+template <int S>
+DEV c2 det_sym_f2(const float2 (&n)[S * (S + 1) / 2]) {
+    auto at = [](int i, int j) { return i * S - i * (i - 1) / 2 + (j - i); }; /* i <= j */
+    const float2 one = bc2(1.f), rt1 = bc2(qmc_secf.one);
+    auto add_rn = [&](float2 a, float2 b) { return fma2(a, rt1, b); };
+    c2 N[S * (S + 1) / 2];
+    {
+        const float2 m2 = fma2(n[0], n[0], one);
+        const float2 d = make_float2(__fdividef(1.f, m2.x), __fdividef(1.f, m2.y));
+        const float2 iy = neg2(mul2(n[0], d)); /* 1 / (1 + i n_0) = d + i iy */
+#pragma unroll
+        for (int i = 1; i < S; ++i) {
+            const float2 u = mul2(n[at(0, i)], iy), v = mul2(n[at(0, i)], d); /* row 0 over the pivot: -u + i v */
+#pragma unroll
+            for (int j = i; j < S; ++j) {
+                const float2 p = mul2(v, n[at(0, j)]);
+                N[at(i, j)] = c2{i == j ? add_rn(p, one) : p, add_rn(n[at(i, j)], mul2(u, n[at(0, j)]))};
+            }
+        }
+    }
+    /* (1 + i n_0) times the second pivot */
+    c2 det = c2{add_rn(N[at(1, 1)].re, neg2(mul2(n[0], N[at(1, 1)].im))), add_rn(N[at(1, 1)].im, mul2(n[0], N[at(1, 1)].re))};
+#pragma unroll
+    for (int k = 1; k < S; ++k) {
+        const c2 dk = N[at(k, k)];
+        if (k > 1) det = cmul2(det, dk);
+        if (k + 1 < S) {
+            const c2 iv = cinv2(dk);
+            const float2 mx = neg2(iv.re), my = neg2(iv.im);
+#pragma unroll
+            for (int i = k + 1; i < S; ++i) {
+                const c2 a = N[at(k, i)];
+                /* l = -a / d_k and m = -Im l */
+                const c2 l = c2{fma2(a.re, mx, mul2(a.im, iv.im)), fma2(a.re, my, mul2(a.im, mx))};
+                const float2 m = fma2(a.re, iv.im, mul2(a.im, iv.re));
+#pragma unroll
+                for (int j = i; j < S; ++j) {
+                    const c2 w = N[at(k, j)];
+                    N[at(i, j)].re = add_rn(N[at(i, j)].re, fma2(l.re, w.re, mul2(m, w.im)));
+                    N[at(i, j)].im = add2(N[at(i, j)].im, fma2(l.re, w.im, mul2(l.im, w.re)));
+                }
+            }
+        }
+    }
+    return det;
+}
+
+/* det_deform_f per lane for S <= 3, in packed arithmetic */
+template <int S>
+DEV c2 det_deform_f2(const float2 (&A)[S][S], float lam) {
+    const float2 l = bc2(lam), ml = bc2(-lam);
+    if constexpr (S == 1) {
+        return c2{bc2(1.f), mul2(ml, A[0][0])};
+    } else if constexpr (S == 2) {
+        const float2 tr = add2(A[0][0], A[1][1]);
+        const float2 dt = fma2(A[0][0], A[1][1], neg2(mul2(A[0][1], A[1][0])));
+        return c2{fma2(mul2(ml, l), dt, bc2(1.f)), mul2(ml, tr)};
+    } else {
+        const float2 tr = add2(add2(A[0][0], A[1][1]), A[2][2]);
+        const float2 p01 = fma2(A[0][0], A[1][1], neg2(mul2(A[0][1], A[1][0])));
+        const float2 p02 = fma2(A[0][0], A[2][2], neg2(mul2(A[0][2], A[2][0])));
+        const float2 p12 = fma2(A[1][1], A[2][2], neg2(mul2(A[1][2], A[2][1])));
+        const float2 e2 = add2(add2(p01, p02), p12);
+        const float2 q1 = fma2(A[1][0], A[2][2], neg2(mul2(A[1][2], A[2][0])));
+        const float2 q2 = fma2(A[1][0], A[2][1], neg2(mul2(A[1][1], A[2][0])));
+        const float2 dt = fma2(A[0][2], q2, fma2(A[0][0], p12, neg2(mul2(A[0][1], q1))));
+        const float2 l2 = mul2(l, l);
+        return c2{fma2(neg2(l2), e2, bc2(1.f)), fma2(mul2(l2, l), dt, mul2(ml, tr))};
+    }
+}
+
+/* G at the points tt of both lanes (eval_G_f per lane): its eps^0 value G0 and, with needX, the eps-coefficient X of
+   its logarithm.  First the undeformed class, where everything is real. */
+template <int S, class Pol>
+DEV void eval_G_f2(const PackedSector &s, const Pol &P, unsigned Y, const float2 *tt, const float2 *Lt, bool needX,
+                   const Exps &ex, float2 &G0, float2 &X) {
+    float2 U, F;
+    P.UFr(Y, tt, U, F);
+    if (s.kind == 1) F = neg2(F);
+    float2 g = bc2(s.Df);
+    if (ex.eU0 != 0) g = mul2(g, rpow2(U, ex.eU0));
+    if (ex.eF0 != 0) g = mul2(g, rpow2(F, -ex.eF0));
+    G0 = mono2<S>(s, g, tt);
+    X = bc2(0.f);
+    if (needX) {
+        float2 a = ex.eU1 != 0 ? rpow2(U, ex.eU1) : bc2(1.f);
+        if (ex.eF1 != 0) a = mul2(a, rpow2(F, -ex.eF1));
+        X = make_float2(__logf(a.x), __logf(a.y));
 #pragma unroll
         for (int j = 0; j < S; ++j)
-            for (int k = 0; k < s.A[j]; ++k) g = mul2(g, tt[j]);
-        G0 = c2{g, bc2(0.f)};
-        X = zero_c2();
-        if (MAXM > 0 && M > 0) {
-            const float2 a = mul2(ipow2(U, ex.eU1), ipow2(F, -ex.eF1));
-            float2 x = make_float2(__logf(a.x), __logf(a.y));
-#pragma unroll
-            for (int j = 0; j < S; ++j)
-                if (s.A[j] != -1 && s.B[j] != 0) x = fma2(bc2((float)s.B[j]), Lt[j], x);
-            X = c2{x, bc2(0.f)};
-        }
-    } else {
-        float2 g[S], h[S * (S + 1) / 2];
+            if ((qmc_secf.l >> j) & 1u) X = fma2(bc2(qmc_secf.B[j]), Lt[j], X);
+    }
+}
+
+/* Deformed sectors, first half: the contour of Eq. 14 at the points tt of both lanes, z_j = t_j (1 - i d_j) with
+   d_j = lam (1 - t_j) dF/dt_j, and its Jacobian. */
+template <int S, class Pol>
+DEV void deform_f2(const Pol &P, unsigned Y, const float2 *tt, const float2 *ttm, float lam, float2 *g, c2 &detJ) {
+    {
+        float2 h[S * (S + 1) / 2];
         P.GH(Y, tt, g, h);
-        cf dets[2];
         if constexpr (S >= 4) {
-            /* the matrix entries of both lanes in packed form (rounded as eval_G_f rounds them), then the
-               elimination per lane with the lane fixed at compile time (no per-element lane selects) */
             float2 sq[S];
 #pragma unroll
             for (int j = 0; j < S; ++j) {
                 const float2 pj = mul2(tt[j], ttm[j]);
                 sq[j] = make_float2(pj.x > 0.f ? pj.x * rsqrtf(pj.x) : 0.f, pj.y > 0.f ? pj.y * rsqrtf(pj.y) : 0.f);
             }
-            float2 bm[S * (S + 1) / 2];
+            const float2 ml = bc2(-lam);
             int p = 0;
 #pragma unroll
             for (int j = 0; j < S; ++j) {
 #pragma unroll
                 for (int i = j; i < S; ++i) {
-                    bm[p] = (i == j) ? fma2(sub2(ttm[j], tt[j]), g[j], mul2(mul2(tt[j], ttm[j]), h[p]))
-                                     : mul2(mul2(sq[j], sq[i]), h[p]);
+                    h[p] = mul2(ml, (i == j) ? fma2(sub2(ttm[j], tt[j]), g[j], mul2(mul2(tt[j], ttm[j]), h[p]))
+                                                : mul2(mul2(sq[j], sq[i]), h[p]));
+                    ++p;
+                }
+            }
+            detJ = det_sym_f2<S>(h);
+        } else {
+            float2 A[S][S];
+            int p = 0;
+#pragma unroll
+            for (int j = 0; j < S; ++j) {
+#pragma unroll
+                for (int i = j; i < S; ++i) {
+                    A[j][i] = mul2(mul2(tt[j], ttm[j]), h[p]);
+                    if (i != j) A[i][j] = mul2(mul2(tt[i], ttm[i]), h[p]);
                     ++p;
                 }
             }
 #pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                cf N[S * (S + 1) / 2];
-                int q = 0;
-#pragma unroll
-                for (int j = 0; j < S; ++j) {
-#pragma unroll
-                    for (int i = j; i < S; ++i) {
-                        N[q] = mkf(i == j ? 1.f : 0.f, -lam * (k ? bm[q].y : bm[q].x));
-                        ++q;
-                    }
-                }
-                dets[k] = det_sym_f<S>(N);
-            }
-        } else {
-#pragma unroll 1
-            for (int k = 0; k < 2; ++k) {
-                /* the determinant per lane, as eval_G_f computes it (one lane at a time: registers) */
-                float A[S][S];
-                int p = 0;
-#pragma unroll
-                for (int j = 0; j < S; ++j) {
-#pragma unroll
-                    for (int i = j; i < S; ++i) {
-                        A[j][i] = lane(tt[j], k) * lane(ttm[j], k) * lane(h[p], k);
-                        if (i != j) A[i][j] = lane(tt[i], k) * lane(ttm[i], k) * lane(h[p], k);
-                        ++p;
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < S; ++j)
-                    A[j][j] = fmaf(lane(ttm[j], k) - lane(tt[j], k), lane(g[j], k), A[j][j]);
-                dets[k] = det_deform_f<S>(A, lam);
-            }
+            for (int j = 0; j < S; ++j) A[j][j] = fma2(sub2(ttm[j], tt[j]), g[j], A[j][j]);
+            detJ = det_deform_f2<S>(A, lam);
         }
-        const c2 detJ = join_c(dets[0], dets[1]);
-        c2 z[S], q[S];
+    }
+#pragma unroll
+    for (int j = 0; j < S; ++j) g[j] = mul2(mul2(bc2(lam), ttm[j]), g[j]);
+}
+
+/* Second half: G at the deformed points.  live: lanes whose point is evaluated (a sign failure is counted only there). */
+template <int S, class Pol>
+DEV void value_f2(const PackedSector &s, const Pol &P, unsigned Y, const float2 *tt, const float2 *g, c2 detJ, bool needX,
+                  const Exps &ex, const bool (&live)[2], c2 &G0, c2 &X, uint32_t &fails) {
+    c2 z[S];
+#pragma unroll
+    for (int j = 0; j < S; ++j) z[j] = c2{tt[j], neg2(mul2(tt[j], g[j]))};
+    c2 U, F;
+    P.UFc(Y, z, ex.eU0 != 0 || needX, U, F);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const float fr = lane(F.re, k), fi = lane(F.im, k);
+        fails += (live[k] && fi > QMC_F32_SIGN_NOISE * (fabsf(fr) + fabsf(fi))) ? 1u : 0u;
+    }
+    c2 G = cscale2(detJ, bc2(s.Df));
+    if (ex.eU0 != 0) G = cmul2(G, cpow2(U, ex.eU0));
+    if (ex.eF0 != 0) G = cmul2(G, cpow2(F, -ex.eF0));
+    if (qmc_secf.a) {
+        if (qmc_secf.a1) G = cscale2(G, mono2<S>(s, bc2(1.f), tt));
+#pragma unroll
+        for (int j = 0; j < S; ++j)
+            if ((qmc_secf.a >> j) & 1u) G = cmul2(G, cpow2(c2{bc2(1.f), neg2(g[j])}, s.A[j]));
+    }
+    G0 = G;
+    X = zero_c2();
+    if (needX) {
+        const float2 eU1 = bc2((float)ex.eU1), eF1 = bc2((float)ex.eF1);
+        const float2 U2 = fma2(U.re, U.re, mul2(U.im, U.im)), F2 = fma2(F.re, F.re, mul2(F.im, F.im));
+        const float2 lU = make_float2(0.5f * __logf(U2.x), 0.5f * __logf(U2.y));
+        const float2 lF = make_float2(0.5f * __logf(F2.x), 0.5f * __logf(F2.y));
+        const float2 aU = make_float2(atan2f(U.im.x, U.re.x), atan2f(U.im.y, U.re.y));
+        const float2 aF = make_float2(arg_mi0f(F.re.x, F.im.x), arg_mi0f(F.re.y, F.im.y));
+        float2 xr = sub2(mul2(lU, eU1), mul2(lF, eF1)), xi = sub2(mul2(aU, eU1), mul2(aF, eF1));
+        /* log q_j with q_j = 1 - i d_j: (log(1 + d_j^2) / 2, -atan d_j) */
+        float2 lr = bc2(0.f);
 #pragma unroll
         for (int j = 0; j < S; ++j) {
-            const float2 d = mul2(mul2(bc2(lam), ttm[j]), g[j]);
-            z[j] = c2{tt[j], neg2(mul2(tt[j], d))};
-            q[j] = c2{bc2(1.f), neg2(d)};
-        }
-        const bool needU = ex.eU0 != 0 || (MAXM > 0 && M > 0);
-        c2 U, F;
-        P.UFc(Y, z, needU, U, F);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float fr = lane(F.re, k), fi = lane(F.im, k);
-            fails += (live[k] && fi > QMC_F32_SIGN_NOISE * (fabsf(fr) + fabsf(fi))) ? 1u : 0u;
-        }
-        c2 G = cscale2(detJ, D);
-        if (ex.eU0 != 0) G = cmul2(G, cipow2(U, ex.eU0));
-        G = cmul2(G, cipow2(F, -ex.eF0));
-        bool any_mono = false;
-        float2 mono = bc2(1.f);
-#pragma unroll
-        for (int j = 0; j < S; ++j)
-            for (int k = 0; k < s.A[j]; ++k) {
-                mono = mul2(mono, tt[j]);
-                any_mono = true;
+            if ((qmc_secf.b >> j) & 1u) {
+                const float2 Bj = bc2(qmc_secf.B[j]), d = g[j];
+                if ((qmc_secf.l >> j) & 1u) xr = fma2(Bj, make_float2(__logf(tt[j].x), __logf(tt[j].y)), xr);
+                const float2 q2 = fma2(d, d, bc2(1.f));
+                lr = fma2(Bj, make_float2(__logf(q2.x), __logf(q2.y)), lr);
+                xi = fma2(neg2(Bj), make_float2(atanf(d.x), atanf(d.y)), xi);
             }
-        if (any_mono) G = cscale2(G, mono);
+        }
+        X = c2{fma2(bc2(0.5f), lr, xr), xi};
+    }
+}
+
+/* Series values of the two classes: real pairs and complex pairs */
+DEV float2 vzero2(float2) { return bc2(0.f); }
+DEV c2 vzero2(c2) { return zero_c2(); }
+DEV float2 vmadd2(float2 o, float2 g, float2 V) { return add2(o, mul2(g, V)); }
+DEV c2 vmadd2(c2 o, c2 g, float2 V) { return cadd2(o, cscale2(g, V)); }
+DEV float2 vnext2(float2 g, float2 X) { return mul2(g, X); }
+DEV c2 vnext2(c2 g, c2 X) { return cmul2(g, X); }
+DEV float2 vscale2(float2 g, float f) { return mul2(g, bc2(f)); }
+DEV c2 vscale2(c2 g, float f) { return cscale2(g, bc2(f)); }
+DEV c2 to_c2(float2 v) { return c2{v, bc2(0.f)}; }
+DEV c2 to_c2(c2 v) { return v; }
+
+/* V times the factor of a singular variable (subset_factor of the FP64 path), for series up to eps^M; a: the variable's
+   series, with 1/B in the place of eps^0 */
+template <int M, int N>
+DEV void subset_factor2(float2 (&V)[N], const float2 *a, bool inY) {
+    float2 f[M + 1];
+    f[0] = inY ? a[0] : bc2(0.f);
 #pragma unroll
-        for (int j = 0; j < S; ++j)
-            if (s.A[j] != 0) G = cmul2(G, cipow2(q[j], s.A[j]));
-        G0 = G;
-        X = zero_c2();
-        if (MAXM > 0 && M > 0) {
-            cf xs[2];
-#pragma unroll 1
-            for (int k = 0; k < 2; ++k) {
-                cf x = csubf(cscalef(clogf_p(lane_c(U, k)), (float)ex.eU1), cscalef(clogf_mi0(lane_c(F, k)), (float)ex.eF1));
-                float lr = 0.f;
+    for (int n = 1; n <= M; ++n) f[n] = inY ? neg2(a[n]) : a[n];
 #pragma unroll
-                for (int j = 0; j < S; ++j) {
-                    if (s.B[j] != 0) {
-                        const float Bj = (float)s.B[j];
-                        if (s.A[j] != -1) x.x = fmaf(Bj, lane(Lt[j], k), x.x);
-                        const float d = -lane(q[j].im, k);
-                        lr = fmaf(Bj, __logf(fmaf(d, d, 1.f)), lr);
-                        x.y = fmaf(-Bj, atanf(d), x.y);
-                    }
-                }
-                x.x = fmaf(0.5f, lr, x.x);
-                xs[k] = x;
-            }
-            X = join_c(xs[0], xs[1]);
+    for (int n = M; n >= 0; --n) {
+        float2 acc = bc2(0.f);
+#pragma unroll
+        for (int k = 0; k <= n; ++k) acc = fma2(V[k], f[n - k], acc);
+        V[n] = acc;
+    }
+}
+
+/* o += G_Y(eps) V_Y(eps) for the subset with the bits `count`, series up to eps^M: V_Y from the shared product `pre` of
+   the first np variables and the factors of the others */
+template <int M, int N, class V2>
+DEV void subset_add2(V2 (&o)[N], V2 g, V2 X, const float2 (&pre)[N], int np, int sigma, unsigned count,
+                     const float2 (*a)[N], int need) {
+    float2 V[N];
+#pragma unroll
+    for (int n = 0; n <= M; ++n) V[n] = pre[n];
+    for (int i = np; i < sigma; ++i) subset_factor2<M>(V, a[i], (count >> i) & 1u);
+#pragma unroll
+    for (int n = 0; n <= M; ++n) {
+        if (n > need) break;
+#pragma unroll
+        for (int k = 0; k + n <= M; ++k) o[n + k] = vmadd2(o[n + k], g, V[k]);
+        if (n < M) {
+            g = vnext2(g, X);
+            if (n > 0) g = vscale2(g, 1.f / (n + 1));
         }
     }
 }
 
-/* w(x) * (sector integrand) at the points (x, y = 1 - x) of both lanes, as point_integrand_f per lane; live[k]:
-   lane k holds a lattice point (its value is zero otherwise) */
-template <int S, bool DEF, int MAXM, class Pol>
-DEV void point_integrand_f2(const PackedSector &s, const Pol &P, const float2 *x, const float2 *y, int r, float lam,
-                            const Exps &ex, bool (&live)[2], c2 (&out)[MAXM + 1], uint32_t &fails) {
-    float2 t[S], tm[S], w = bc2(1.f);
+template <int MAXM, class V2>
+DEV void subset_add2(int M, V2 (&o)[MAXM + 1], V2 g, V2 X, const float2 (&pre)[MAXM + 1], int np, int sigma, unsigned count,
+                     const float2 (*a)[MAXM + 1], int need) {
+    switch (MAXM == 0 ? 0 : M) {
+        case 0: subset_add2<0>(o, g, X, pre, np, sigma, count, a, need); break;
+        case 1: if constexpr (MAXM >= 1) subset_add2<1>(o, g, X, pre, np, sigma, count, a, need); break;
+        case 2: if constexpr (MAXM >= 2) subset_add2<2>(o, g, X, pre, np, sigma, count, a, need); break;
+        case 3: if constexpr (MAXM >= 3) subset_add2<3>(o, g, X, pre, np, sigma, count, a, need); break;
+        case 4: if constexpr (MAXM >= 4) subset_add2<4>(o, g, X, pre, np, sigma, count, a, need); break;
+        default: break;
+    }
+}
+
+/* The transform of both lanes' points (x, y = 1 - x); live[k]: lane k holds a lattice point, and on return whether its
+   weight is positive.  A lane without a point takes the other lane's (its value is discarded).  false: neither lane. */
+template <int S>
+DEV bool pair_setup(const float2 *x, const float2 *y, int r, bool (&live)[2], float2 (&t)[S], float2 (&tm)[S], float2 &w) {
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         float2 wj;
         transform2(r, x[j], y[j], t[j], tm[j], wj);
-        w = mul2(w, wj);
+        w = j == 0 ? wj : mul2(w, wj);
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
@@ -2080,10 +2227,7 @@ DEV void point_integrand_f2(const PackedSector &s, const Pol &P, const float2 *x
         for (int j = 0; j < S; ++j) bad |= !(lane(t[j], k) > 0.f) || !(lane(tm[j], k) > 0.f);
         live[k] = live[k] && !bad;
     }
-#pragma unroll
-    for (int n = 0; n <= MAXM; ++n) out[n] = zero_c2();
-    if (!live[0] && !live[1]) return;
-    /* a lane without a point evaluates the other lane's point; its value is discarded */
+    if (!live[0] && !live[1]) return false;
     if (!live[0] || !live[1]) {
         const int from = live[0] ? 0 : 1;
 #pragma unroll
@@ -2093,17 +2237,76 @@ DEV void point_integrand_f2(const PackedSector &s, const Pol &P, const float2 *x
         }
         w = bc2(lane(w, from));
     }
+    return true;
+}
+
+/* logarithms of the variables that need one, and the series eps t^{-1 + B eps} of the singular ones */
+template <int S, int MAXM>
+DEV void pair_series(const PackedSector &s, const float2 (&t)[S], float2 (&Lt)[S], float2 (&a)[S][MAXM + 1]) {
     const int M = s.M;
-    const unsigned smask = (unsigned)s.sing_mask;
-    float2 Lt[S];
+    int i = 0;
 #pragma unroll
-    for (int j = 0; j < S; ++j) Lt[j] = bc2(0.f);
-    if (MAXM > 0 && M > 0) {
+    for (int j = 0; j < S; ++j) {
+        const bool sing = ((unsigned)s.sing_mask >> j) & 1u;
+        Lt[j] = bc2(0.f);
+        if (MAXM > 0 && M > 0 && (sing || ((qmc_secf.l >> j) & 1u))) Lt[j] = make_float2(__logf(t[j].x), __logf(t[j].y));
+        if (!sing) continue;
+        a[i][0] = bc2(qmc_secf.rB[j]); /* the place of eps^0 holds 1/B_j */
+        if (MAXM > 0 && M > 0) {
+            float2 c = make_float2(__fdividef(1.f, t[j].x), __fdividef(1.f, t[j].y));
+            const float2 bl = mul2(bc2(qmc_secf.B[j]), Lt[j]);
 #pragma unroll
-        for (int j = 0; j < S; ++j)
-            if (((smask >> j) & 1u) || s.B[j] != 0) Lt[j] = make_float2(__logf(t[j].x), __logf(t[j].y));
+            for (int n = 1; n <= MAXM; ++n) {
+                a[i][n] = c;
+                if (n >= M) break;
+                c = mul2(c, n == 1 ? bl : make_float2(bl.x / n, bl.y / n));
+            }
+        }
+        ++i;
     }
-    unsigned Y = 0;
+}
+
+/* w(x) * (sector integrand) at the points (x, y = 1 - x) of both lanes, as point_integrand_f per lane; live[k]:
+   lane k holds a lattice point (its value is zero otherwise).
+   As in the FP64 path, the series of the singular variables and the products of all but the last of them are made once
+   per pair of points (local memory), and G_Y is taken only to the order at which its subset contributes: what is left
+   out are sums and products with exact zeros, and logarithms that nothing uses.  Bound by instruction issue; with the
+   same point values, mixed passes (16 shifts): massive box n = 1048573 1.05 -> 0.86 ms, four-pole double box n = 65521
+   (all FP32) 12.4 -> 9.1 ms. */
+template <int S, bool DEF, int MAXM, class Pol>
+DEV void point_integrand_f2(const PackedSector &s, const Pol &P, const float2 *x, const float2 *y, int r, float lam,
+                            const Exps &ex, bool (&live)[2], c2 (&out)[MAXM + 1], uint32_t &fails) {
+    typedef typename Select<DEF, c2, float2>::type V2;
+    float2 t[S], tm[S], w;
+#pragma unroll
+    for (int n = 0; n <= MAXM; ++n) out[n] = zero_c2();
+    if (!pair_setup<S>(x, y, r, live, t, tm, w)) return;
+    const int M = s.M, sigma = s.sigma;
+    const unsigned smask = (unsigned)s.sing_mask;
+    float2 Lt[S], a[S][MAXM + 1];
+    pair_series<S, MAXM>(s, t, Lt, a);
+    constexpr int NPRE = S < 4 ? S : 4;
+    float2 pre[1 << (NPRE - 1)][MAXM + 1];
+    const int np = sigma < NPRE ? (sigma > 0 ? sigma - 1 : 0) : NPRE - 1;
+#pragma unroll
+    for (int n = 0; n <= MAXM; ++n) pre[0][n] = bc2(n == 0 ? 1.f : 0.f);
+    for (int i = 0; i < np; ++i)
+        for (int k = 0; k < (1 << i); ++k) {
+            float2 V[MAXM + 1], W[MAXM + 1];
+#pragma unroll
+            for (int n = 0; n <= MAXM; ++n) V[n] = W[n] = pre[k][n];
+            subset_factor2<MAXM>(V, a[i], false);
+            subset_factor2<MAXM>(W, a[i], true);
+#pragma unroll
+            for (int n = 0; n <= MAXM; ++n) {
+                pre[k][n] = V[n];
+                pre[k + (1 << i)][n] = W[n];
+            }
+        }
+    V2 o[MAXM + 1];
+#pragma unroll
+    for (int n = 0; n <= MAXM; ++n) o[n] = vzero2(o[n]);
+    unsigned Y = 0, count = 0;
     do {
         float2 tt[S], ttm[S];
 #pragma unroll
@@ -2112,50 +2315,23 @@ DEV void point_integrand_f2(const PackedSector &s, const Pol &P, const float2 *x
             tt[j] = zj ? bc2(0.f) : t[j];
             ttm[j] = zj ? bc2(1.f) : tm[j];
         }
-        c2 G0, X;
-        eval_G_f2<S, DEF, MAXM>(s, P, Y, tt, ttm, Lt, lam, M, ex, live, G0, X, fails);
-        float2 V[MAXM + 1];
-        V[0] = bc2(1.f);
-#pragma unroll
-        for (int n = 1; n <= MAXM; ++n) V[n] = bc2(0.f);
-#pragma unroll
-        for (int j = 0; j < S; ++j) {
-            if ((smask >> j) & 1u) {
-                const bool inY = (Y >> j) & 1u;
-                const float Bj = (float)s.B[j];
-                float2 f[MAXM + 1];
-                f[0] = bc2(inY ? __fdividef(1.f, Bj) : 0.f);
-                float2 c = make_float2(__fdividef(1.f, t[j].x), __fdividef(1.f, t[j].y));
-#pragma unroll
-                for (int n = 1; n <= MAXM; ++n) {
-                    f[n] = inY ? neg2(c) : c;
-                    /* c *= B_j Lt_j / n, per lane as the one-point code */
-                    c = make_float2(c.x * (Bj * Lt[j].x / n), c.y * (Bj * Lt[j].y / n));
-                }
-#pragma unroll
-                for (int n = MAXM; n >= 0; --n) {
-                    float2 acc = bc2(0.f);
-#pragma unroll
-                    for (int k = 0; k <= n; ++k) acc = fma2(V[k], f[n - k], acc);
-                    V[n] = acc;
-                }
-            }
-        }
-        c2 g = G0;
-#pragma unroll
-        for (int n = 0; n <= MAXM; ++n) {
-            if (n <= M) {
-#pragma unroll
-                for (int k = 0; k + n <= MAXM; ++k)
-                    if (n + k <= M) out[n + k] = cadd2(out[n + k], cscale2(g, V[k]));
-                g = cscale2(cmul2(g, X), bc2(1.f / (n + 1)));
-            }
-        }
+        const int need = M - sigma + __popc(count); /* highest order of eps to which G_Y is needed */
+        V2 G0, X;
+        if constexpr (DEF) {
+            float2 d[S];
+            c2 detJ;
+            deform_f2<S>(P, Y, tt, ttm, lam, d, detJ);
+            value_f2<S>(s, P, Y, tt, d, detJ, MAXM > 0 && need > 0, ex, live, G0, X, fails);
+        } else
+            eval_G_f2<S>(s, P, Y, tt, Lt, MAXM > 0 && need > 0, ex, G0, X);
+        const unsigned low = count & ((1u << np) - 1u);
+        subset_add2<MAXM>(M, o, G0, X, pre[low], np, sigma, count, a, need);
+        ++count;
         Y = (Y - smask) & smask;
     } while (Y != 0);
 #pragma unroll
     for (int n = 0; n <= MAXM; ++n) {
-        out[n] = cscale2(out[n], w);
+        out[n] = cscale2(to_c2(o[n]), w);
         if (!live[0]) out[n] = c2{make_float2(0.f, out[n].re.y), make_float2(0.f, out[n].im.y)};
         if (!live[1]) out[n] = c2{make_float2(out[n].re.x, 0.f), make_float2(out[n].im.x, 0.f)};
     }
@@ -2169,12 +2345,118 @@ DEV void stage_sector_f2(const unsigned char *packed, int64_t sectors_off, int64
     int4 *dst = reinterpret_cast<int4 *>(smem);
     constexpr int NS = (int)(sizeof(PackedSector) / 16);
     for (int k = threadIdx.x; k < NS; k += blockDim.x) dst[k] = src[k];
+    if (threadIdx.x < 8) {
+        const float B = (float)ps->B[threadIdx.x];
+        qmc_secf.B[threadIdx.x] = B;
+        qmc_secf.rB[threadIdx.x] = __fdividef(1.f, B); /* used for singular variables only: B != 0 there */
+        const int A = ps->A[threadIdx.x];
+        const unsigned m = 0xffu;
+        const unsigned a1 = __ballot_sync(m, A >= 1), a2 = __ballot_sync(m, A >= 2), more = __ballot_sync(m, A >= 3);
+        const unsigned an = __ballot_sync(m, A != 0), b = __ballot_sync(m, B != 0.f), l = __ballot_sync(m, B != 0.f && A != -1);
+        if (threadIdx.x == 0) {
+            qmc_secf.a1 = a1;
+            qmc_secf.a2 = a2;
+            qmc_secf.more = more;
+            qmc_secf.a = an;
+            qmc_secf.b = b;
+            qmc_secf.l = l;
+            qmc_secf.one = 1.f;
+        }
+    }
     const int nt = ps->n_terms;
     const PackedTermF *tsrc = reinterpret_cast<const PackedTermF *>(packed + termsf_off) + ps->term0;
     float4 *tdst = reinterpret_cast<float4 *>(dst + NS);
     for (int k = threadIdx.x; k < nt; k += blockDim.x) {
         const float hi = tsrc[k].hi, lo = tsrc[k].lo;
         tdst[k] = make_float4(hi, hi, lo, lo);
+    }
+}
+
+/* Points p and p + 1 of the thread whose first lattice index is i0 (stride: threads of the item): coordinates x and 1 - x
+   of both lanes, and which of them are evaluated here; steps the residues r_j past both. */
+template <int S>
+DEV void next_pair(long long i0, int p, int P, int stride, uint32_t n, float invnf, int level, unsigned smask, float rn, float xi,
+                   uint32_t (&rj)[S], const uint32_t (&aj)[S], const float (&bj)[S], const uint32_t (&zs)[S], bool (&live)[2],
+                   float2 (&x)[S], float2 (&y)[S]) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const long long i = i0 + (long long)(p + k) * stride;
+        live[k] = (p + k < P) && i < (long long)n;
+        if (live[k] && level >= 0) {
+            uint32_t kk[S];
+#pragma unroll
+            for (int j = 0; j < S; ++j) kk[j] = shifted_index(rj[j], aj[j], n);
+            live[k] = !(island_key<S>(kk, smask, rn) < xi);
+        }
+#pragma unroll
+        for (int j = 0; j < S; ++j) {
+            float xv, yv;
+            lattice_f32(rj[j], aj[j], bj[j], n, invnf, xv, yv);
+            if (k == 0) {
+                x[j].x = xv;
+                y[j].x = yv;
+            } else {
+                x[j].y = xv;
+                y[j].y = yv;
+            }
+            const uint32_t v = rj[j] + zs[j];
+            rj[j] = v >= n ? v - n : v;
+        }
+    }
+}
+
+/* adds both lanes' values to a thread's sums, lane a first */
+template <int MAXM>
+DEV void add_pair(float (&acc)[2 * (MAXM + 1)], float (&cmp)[2 * (MAXM + 1)], const c2 (&val)[MAXM + 1], const bool (&live)[2]) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (!live[k]) continue;
+#pragma unroll
+        for (int m = 0; m <= MAXM; ++m) {
+            two_sum_acc(acc[2 * m], cmp[2 * m], lane(val[m].re, k));
+            two_sum_acc(acc[2 * m + 1], cmp[2 * m + 1], lane(val[m].im, k));
+        }
+    }
+}
+
+/* a warp's sums: double-float shuffle tree; s_red, s_fail: the warp's place */
+template <int MAXM>
+DEV void warp_sums(const float (&acc)[2 * (MAXM + 1)], const float (&cmp)[2 * (MAXM + 1)], uint32_t fails, double *s_red,
+                   uint32_t *s_fail) {
+    const int lane_id = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < 2 * (MAXM + 1); ++q) {
+        float s1 = acc[q], c1 = cmp[q];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const float so = __shfl_down_sync(0xffffffffu, s1, off);
+            const float co = __shfl_down_sync(0xffffffffu, c1, off);
+            two_sum_acc(s1, c1, so);
+            c1 += co;
+        }
+        if (lane_id == 0) s_red[q] = (double)s1 + (double)c1;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) fails += __shfl_down_sync(0xffffffffu, fails, off);
+    if (lane_id == 0) *s_fail = fails;
+}
+
+/* an item's partial from its warps' sums (compensated, in order), written by the item's first 32 threads (q: thread);
+   add: to what the FP64 kernel left there for the island points */
+template <int MAXM>
+DEV void write_partial(const Job &J, long long local, int q, const double (*s_red)[2 * (MAXM + 1)], const uint32_t *s_fail,
+                       int nwarps, bool add) {
+    if (q < J.n_slots * 2) {
+        double s2 = 0.0, c2v = 0.0;
+        if (q < 2 * (MAXM + 1))
+            for (int w = 0; w < nwarps; ++w) kahan_add(s2, c2v, s_red[w][q]);
+        double *dst = &J.partials[local * J.n_slots * 2 + q];
+        *dst = add ? *dst + (s2 - c2v) : s2 - c2v;
+    }
+    if (q == 0) {
+        uint32_t tf = 0;
+        for (int w = 0; w < nwarps; ++w) tf += s_fail[w];
+        J.part_fails[local] = add ? J.part_fails[local] + tf : tf;
     }
 }
 
@@ -2190,7 +2472,7 @@ DEV void eval_f32x2_body(const JobTable &jt) {
     __shared__ uint32_t s_fail[16];
     const PackedSector &sec = *reinterpret_cast<const PackedSector *>(smem);
     const float4 *T = reinterpret_cast<const float4 *>(smem + sizeof(PackedSector));
-    const int lane_id = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     int cur = -1, cur_job = -1;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -2233,7 +2515,7 @@ DEV void eval_f32x2_body(const JobTable &jt) {
             cur = psec;
             cur_job = jb;
         }
-        const Exps ex{J.eU0, J.eU1, J.eF0, J.eF1};
+        const Exps ex = Pol::exps(J);
         const Pol pol = Pol::make(T, sec, psec);
         const uint32_t n = J.n;
         const float invnf = 1.f / (float)n;
@@ -2255,77 +2537,208 @@ DEV void eval_f32x2_body(const JobTable &jt) {
         for (int p = 0; p < jt.P; p += 2) {
             bool live[2];
             float2 x[S], y[S];
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const long long i = i0 + (long long)(p + k) * blockDim.x;
-                live[k] = (p + k < jt.P) && i < (long long)n;
-                if (live[k] && level >= 0) {
-                    uint32_t kk[S];
-#pragma unroll
-                    for (int j = 0; j < S; ++j) kk[j] = shifted_index(rj[j], aj[j], n);
-                    live[k] = !(island_key<S>(kk, (unsigned)sec.sing_mask, rn) < xi);
-                }
-#pragma unroll
-                for (int j = 0; j < S; ++j) {
-                    float xv, yv;
-                    lattice_f32(rj[j], aj[j], bj[j], n, invnf, xv, yv);
-                    if (k == 0) {
-                        x[j].x = xv;
-                        y[j].x = yv;
-                    } else {
-                        x[j].y = xv;
-                        y[j].y = yv;
-                    }
-                    const uint32_t v = rj[j] + zs[j];
-                    rj[j] = v >= n ? v - n : v;
-                }
-            }
+            next_pair<S>(i0, p, jt.P, blockDim.x, n, invnf, level, (unsigned)sec.sing_mask, rn, xi, rj, aj, bj, zs, live, x, y);
             if (live[0] || live[1]) {
                 c2 val[MAXM + 1];
                 point_integrand_f2<S, DEF, MAXM>(sec, pol, x, y, jt.r, lam, ex, live, val, fails);
+                add_pair<MAXM>(acc, cmp, val, live);
+            }
+        }
+        warp_sums<MAXM>(acc, cmp, fails, s_red[warp], &s_fail[warp]);
+        __syncthreads();
+        if (threadIdx.x < 32) write_partial<MAXM>(J, local, threadIdx.x, s_red, s_fail, nwarps, level >= 0);
+        __syncthreads();
+    }
+}
+
+/* ------------------------------------------------------------------ K2x2 in phases: deformed sectors of 5 and 6 dimensions
+ * A pair of points of such a sector runs through 2400 instructions per zeroed subset, 38 KB of straight-line code of
+ * which nothing repeats.  An SM partition issues one instruction per cycle from a 32 KB instruction cache, 0.4 per warp
+ * from the next level and 0.17 from L2 (measured with loops of 2 KB to 256 KB): with three independent blocks per SM a
+ * warp spent 2.5 of 6.8 cycles per instruction waiting for instructions, and more where the blocks were in different
+ * sectors.  So all sixteen warps of an SM form one block that goes through the code in two phases per subset, each
+ * short enough for that cache (contour and Jacobian; value and accumulation), over `pairs` pairs of points per thread,
+ * with a barrier between them: a phase's code is fetched once for 4 warps x `pairs` passes.  What a pair carries from
+ * phase to phase (coordinates, contour, Jacobian, series: 26 packed pairs for S = 6, MAXM = 2) lies in shared memory,
+ * 208 bytes per pair and thread.  The block works on consecutive items of one sector, one per group of jt.block threads
+ * (the threads of an item in the other kernels), so that items, their partials and their order of summation are those
+ * of every other kernel.  item_begin and total_items count such sets of items here.
+ * Measured (16 shifts), determinant per lane with three blocks per SM -> packed determinant and shorter series
+ * with three blocks -> in phases: non-planar double box n = 3001 0.78, 0.71 -> 0.46 ms, n = 16381 2.1 -> 1.85 ms,
+ * n = 1048573 115.7, 98-100 -> 103.0 ms; planar double box n = 50021 6.98, 5.92 -> 4.87 ms: three blocks stay 3 % ahead
+ * only where every block is in the same sector for long.  What bounds it now is the FP32 pipe's operand ports: a packed
+ * FMA with three distinct register pairs takes 3 cycles of a partition, a packed product 2; some 3000 cycles of 5200
+ * per pair and subset.  384 threads, one pair in flight, or a barrier after the second phase: 0 to 9 % slower. */
+template <int S, int MAXM>
+struct PairState {
+    enum { T = 0, TM = S, D = 2 * S, DET = 3 * S, O = 3 * S + 2, SIZE = 3 * S + 2 + 2 * (MAXM + 1) };
+};
+
+template <int S, int MAXM, class Pol>
+DEV void eval_f32x2_phased_body(const JobTable &jt) {
+    typedef PairState<S, MAXM> PS;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ long long s_item;
+    __shared__ int s_job, s_abort;
+    __shared__ double s_red[QMC_PHASED_THREADS / 32][2 * (MAXM + 1)];
+    __shared__ uint32_t s_fail[QMC_PHASED_THREADS / 32];
+    const PackedSector &sec = *reinterpret_cast<const PackedSector *>(smem);
+    const float4 *T = reinterpret_cast<const float4 *>(smem + sizeof(PackedSector));
+    float2 *state = reinterpret_cast<float2 *>(smem + jt.state_off) + threadIdx.x; /* [pair][value][thread] */
+    const int stride = jt.block, groups = QMC_PHASED_THREADS / stride;
+    const int group = threadIdx.x / stride, tl = threadIdx.x - group * stride;
+    const int warp = threadIdx.x >> 5, nwarps = stride >> 5;
+    auto st = [&](int q, int k) -> float2 & { return state[(q * PS::SIZE + k) * QMC_PHASED_THREADS]; };
+    int cur = -1, cur_job = -1;
+    for (;;) {
+        if (threadIdx.x == 0) {
+            const long long it = (long long)atomicAdd(jt.counter, 1ull);
+            s_item = it;
+            s_job = it < jt.total_items ? find_job(jt, it) : 0;
+            s_abort = it < jt.total_items ? job_aborted(jt.jobs[s_job]) : 0;
+        }
+        __syncthreads();
+        if (s_item >= jt.total_items) break;
+        const int jb = s_job;
+        const Job &J = jt.jobs[jb];
+        const long long per_sector = (long long)J.m * J.chunks, sets = (per_sector + groups - 1) / groups;
+        const long long set = s_item - J.item_begin;
+        const int ls = (int)(set / sets);
+        const long long rem = (set - (long long)ls * sets) * groups + group; /* this group's item within the sector */
+        const bool have = group < groups && rem < per_sector; /* groups x jt.block threads may be fewer than the block */
+        const long long local = (long long)ls * per_sector + rem;
+        const int shift = have ? (int)(rem / J.chunks) : 0;
+        const long long chunk = have ? rem - (long long)shift * J.chunks : 0;
+        const int psec = J.sector_begin + ls;
+        if (s_abort) { /* the pass was stopped: its remaining items contribute nothing */
+            if (have && tl < J.n_slots * 2) J.partials[local * J.n_slots * 2 + tl] = 0.0;
+            if (have && tl == 0) J.part_fails[local] = 0;
+            __syncthreads();
+            continue;
+        }
+        int level = -1; /* island level: the FP64 kernel has evaluated the island points and written the partial */
+        if (J.sector_prec) {
+            const PackedSector *gps = reinterpret_cast<const PackedSector *>(J.packed + J.sectors_off) + psec;
+            const int code = J.sector_prec[gps->orig_index];
+            level = island_level(code);
+            if (code != 1 && level < 0) {
+                __syncthreads();
+                continue;
+            }
+        }
+        if (psec != cur || jb != cur_job) {
+            stage_sector_f2(J.packed, J.sectors_off, J.termsf_off, psec, smem);
+            __syncthreads();
+            cur = psec;
+            cur_job = jb;
+        }
+        const Exps ex = Pol::exps(J);
+        const Pol pol = Pol::make(T, sec, psec);
+        const uint32_t n = J.n;
+        const float invnf = 1.f / (float)n;
+        const float lam = (float)J.lambda[sec.orig_index];
+        uint32_t rj[S], aj[S], zs[S];
+        float bj[S];
+        const long long i0 = chunk * (long long)stride * jt.P + tl;
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    if (!live[k]) continue;
+        for (int j = 0; j < S; ++j) {
+            split_shift(J.shifts[6 * shift + j], n, aj[j], bj[j]);
+            rj[j] = (uint32_t)(((unsigned long long)i0 * J.z[j]) % n);
+            zs[j] = J.zstep[j];
+        }
+        float acc[2 * (MAXM + 1)], cmp[2 * (MAXM + 1)];
 #pragma unroll
-                    for (int m = 0; m <= MAXM; ++m) {
-                        two_sum_acc(acc[2 * m], cmp[2 * m], lane(val[m].re, k));
-                        two_sum_acc(acc[2 * m + 1], cmp[2 * m + 1], lane(val[m].im, k));
+        for (int q = 0; q < 2 * (MAXM + 1); ++q) acc[q] = cmp[q] = 0.f;
+        uint32_t fails = 0;
+        const float rn = island_rn(n), xi = island_xi(level < 0 ? 0 : level);
+        const int M = sec.M, sigma = sec.sigma;
+        const unsigned smask = (unsigned)sec.sing_mask;
+        for (int p0 = 0; p0 < jt.P; p0 += 2 * jt.pairs) {
+            unsigned lives = 0; /* two bits per pair */
+            float2 w0 = bc2(0.f), w1 = bc2(0.f); /* weights of the (at most two) pairs */
+            unsigned Y = 0, count = 0;
+            do {
+                const unsigned next = (Y - smask) & smask;
+                for (int q = 0; q < jt.pairs && p0 + 2 * q < jt.P; ++q) {
+                    float2 t[S], tm[S];
+                    if (Y == 0) {
+                        bool live[2];
+                        float2 x[S], y[S], w;
+                        next_pair<S>(i0, p0 + 2 * q, jt.P, stride, n, invnf, level, smask, rn, xi, rj, aj, bj, zs, live, x, y);
+                        live[0] = live[0] && have;
+                        live[1] = live[1] && have;
+                        if (!(live[0] || live[1]) || !pair_setup<S>(x, y, jt.r, live, t, tm, w)) continue;
+                        lives |= (live[0] ? 1u : 0u) << (2 * q) | (live[1] ? 2u : 0u) << (2 * q);
+#pragma unroll
+                        for (int j = 0; j < S; ++j) st(q, PS::T + j) = t[j];
+                        if (smask) {
+#pragma unroll
+                            for (int j = 0; j < S; ++j) st(q, PS::TM + j) = tm[j];
+                        }
+                        if (q == 0) w0 = w;
+                        else w1 = w;
+                    } else {
+                        if (!((lives >> (2 * q)) & 3u)) continue;
+#pragma unroll
+                        for (int j = 0; j < S; ++j) {
+                            const bool zj = (Y >> j) & 1u;
+                            t[j] = zj ? bc2(0.f) : st(q, PS::T + j);
+                            tm[j] = zj ? bc2(1.f) : st(q, PS::TM + j);
+                        }
+                    }
+                    float2 d[S];
+                    c2 detJ;
+                    deform_f2<S>(pol, Y, t, tm, lam, d, detJ);
+#pragma unroll
+                    for (int j = 0; j < S; ++j) st(q, PS::D + j) = d[j];
+                    st(q, PS::DET) = detJ.re;
+                    st(q, PS::DET + 1) = detJ.im;
+                }
+                __syncthreads();
+                for (int q = 0; q < jt.pairs && p0 + 2 * q < jt.P; ++q) {
+                    const unsigned lv = (lives >> (2 * q)) & 3u;
+                    if (!lv) continue;
+                    const bool live[2] = {(lv & 1u) != 0, (lv & 2u) != 0};
+                    float2 t[S], tt[S], d[S];
+#pragma unroll
+                    for (int j = 0; j < S; ++j) {
+                        t[j] = st(q, PS::T + j);
+                        tt[j] = (Y >> j) & 1u ? bc2(0.f) : t[j];
+                        d[j] = st(q, PS::D + j);
+                    }
+                    const int need = M - sigma + __popc(count);
+                    c2 G0, X;
+                    value_f2<S>(sec, pol, Y, tt, d, c2{st(q, PS::DET), st(q, PS::DET + 1)}, MAXM > 0 && need > 0, ex, live, G0, X,
+                                fails);
+                    c2 o[MAXM + 1];
+#pragma unroll
+                    for (int m = 0; m <= MAXM; ++m)
+                        o[m] = count == 0 ? zero_c2() : c2{st(q, PS::O + 2 * m), st(q, PS::O + 2 * m + 1)};
+                    float2 one[MAXM + 1], Lt[S], a[S][MAXM + 1];
+#pragma unroll
+                    for (int m = 0; m <= MAXM; ++m) one[m] = bc2(m == 0 ? 1.f : 0.f);
+                    pair_series<S, MAXM>(sec, t, Lt, a);
+                    subset_add2<MAXM>(M, o, G0, X, one, 0, sigma, count, a, need);
+                    if (next != 0) {
+#pragma unroll
+                        for (int m = 0; m <= MAXM; ++m) {
+                            st(q, PS::O + 2 * m) = o[m].re;
+                            st(q, PS::O + 2 * m + 1) = o[m].im;
+                        }
+                    } else {
+                        const float2 w = q == 0 ? w0 : w1;
+#pragma unroll
+                        for (int m = 0; m <= MAXM; ++m) o[m] = cscale2(o[m], w);
+                        add_pair<MAXM>(acc, cmp, o, live);
                     }
                 }
-            }
+                ++count;
+                Y = next;
+            } while (Y != 0);
         }
-#pragma unroll
-        for (int q = 0; q < 2 * (MAXM + 1); ++q) {
-            float s1 = acc[q], c1 = cmp[q];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                const float so = __shfl_down_sync(0xffffffffu, s1, off);
-                const float co = __shfl_down_sync(0xffffffffu, c1, off);
-                two_sum_acc(s1, c1, so);
-                c1 += co;
-            }
-            if (lane_id == 0) s_red[warp][q] = (double)s1 + (double)c1;
-        }
-        uint32_t f = fails;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) f += __shfl_down_sync(0xffffffffu, f, off);
-        if (lane_id == 0) s_fail[warp] = f;
+        warp_sums<MAXM>(acc, cmp, fails, s_red[warp], &s_fail[warp]);
         __syncthreads();
-        if (threadIdx.x < 32) {
-            const int q = threadIdx.x;
-            if (q < J.n_slots * 2) {
-                double s2 = 0.0, c2v = 0.0;
-                if (q < 2 * (MAXM + 1))
-                    for (int w = 0; w < nwarps; ++w) kahan_add(s2, c2v, s_red[w][q]);
-                double *dst = &J.partials[local * J.n_slots * 2 + q];
-                *dst = level >= 0 ? *dst + (s2 - c2v) : s2 - c2v;
-            }
-            if (q == 0) {
-                uint32_t tf = 0;
-                for (int w = 0; w < nwarps; ++w) tf += s_fail[w];
-                J.part_fails[local] = level >= 0 ? J.part_fails[local] + tf : tf;
-            }
-        }
+        if (have && tl < 32) write_partial<MAXM>(J, local, tl, s_red + group * nwarps, s_fail + group * nwarps, nwarps, level >= 0);
         __syncthreads();
     }
 }

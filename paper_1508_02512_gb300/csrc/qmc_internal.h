@@ -114,7 +114,10 @@ struct JobTable {
     int32_t n_jobs, r, P, want_prec;
     int64_t total_items;
     unsigned long long *counter;  /* work counter of this launch (zeroed before it) */
-    int32_t smem_bytes, pad;
+    int32_t smem_bytes;
+    int32_t block, pairs, state_off; /* phased FP32 kernel: threads of an item, pairs of points in flight per thread, and
+                                        the offset of their state in shared memory */
+    int32_t pad;
     Job jobs[QMC_MAX_JOBS];
 };
 
@@ -195,5 +198,11 @@ int qmc_launch_probe(int dim, int deform, int maxm, const ProbeArgs &a, void *st
 int qmc_gen_kernel(const void *packed_host, int precision, int cls, const void **eval_kernel);
 uint64_t qmc_family_key(const void *packed_host); /* computed from the image, not read from its header */
 int qmc_gen_max_block(int dim);                  /* largest block of a generated kernel for sectors of this dimension */
+/* Whether the generated FP32 kernel of this class works in phases (eval_f32x2_phased_body): then it runs
+   QMC_PHASED_THREADS / block groups of `block` threads per block, each on an item, and needs qmc_phased_state bytes of
+   shared memory per pair of points in flight and thread. */
+#define QMC_PHASED_THREADS 512
+inline bool qmc_gen_phased(int dim, int cls) { return cls == 1 && dim >= 5; }
+inline int qmc_phased_state(int dim, int maxm) { return (3 * dim + 2 + 2 * (maxm + 1)) * 8; }
 int qmc_gen_blocks_per_sm(const void *kernel, int block, int smem_bytes, int *out);
 int qmc_gen_launch_eval(const void *kernel, const JobTable &t, int grid, int block, void *stream);

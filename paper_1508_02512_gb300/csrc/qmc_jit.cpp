@@ -42,7 +42,7 @@
 
 namespace {
 
-#define QMC_JIT_GENERATOR_VERSION 9u
+#define QMC_JIT_GENERATOR_VERSION 11u
 #define QMC_GEN_INLINE_TERMS 2048 /* families with more terms get out-of-line sector functions */
 
 const PackedHeader *hdr(const void *p) {
@@ -77,6 +77,10 @@ uint64_t family_key(const PackedHeader *h) {
     f.add_i(QMC_JIT_GENERATOR_VERSION);
     f.add_i(h->dim);
     f.add_i(h->n_sectors);
+    f.add_i(h->eU0);
+    f.add_i(h->eU1);
+    f.add_i(h->eF0);
+    f.add_i(h->eF1);
     for (int c = 0; c < QMC_N_CLASSES; ++c) {
         f.add_i(h->class_begin[c]);
         f.add_i(h->class_end[c]);
@@ -446,6 +450,9 @@ std::string generate(const PackedHeader *h, const Lang &L) {
     const std::string Pol = L.pol;
     o += "\nstruct " + Pol + " {\n    const " + TT + " *T;\n    int sec;\n    DEV static " + Pol + " make(const " + TT +
          " *T, const PackedSector &, int psec) { return " + Pol + "{T, psec}; }\n";
+    std::snprintf(b, sizeof(b), "    DEV static Exps exps(const Job &) { return Exps{%d, %d, %d, %d}; }\n", h->eU0, h->eU1, h->eF0,
+                  h->eF1);
+    o += b;
     /* case labels: sector * 64 + Y; a sector with one function for all subsets gets the labels of every Y */
     auto labels = [&](int s, unsigned Y) {
         if (per_subset(s) || ps[s].sing_mask == 0) return "case " + std::to_string(s * 64 + (int)Y) + ":";
@@ -496,19 +503,22 @@ std::string generate(const PackedHeader *h, const Lang &L) {
         if (h->class_end[c] <= h->class_begin[c]) continue;
         const char *def = c == 1 ? "true" : "false";
         const int mm = maxm_of(h, c);
-        /* FP32, 5- and 6-dimensional sectors, 128-thread blocks: the deformed class at 3 blocks per SM (<= 170
-           registers, no spills; 13 % faster than 2 blocks, 3 % faster than 4, which spills); the undeformed class
-           at 4 blocks per SM (17 % faster than 3 on the four-pole sectors of the massless double box, which are
-           latency-bound).  FP32 below 5 dimensions: registers capped for 768 threads per SM (the massive box
-           pass is 18 % faster than with the compiler's 125 registers and 512 threads).  FP64 keeps 256. */
-        const std::string lb = L.f64 ? "__launch_bounds__(256)"
-                               : qmc_gen_max_block(S) == 128
-                                   ? (c == 1 ? "__launch_bounds__(128, 3)" : "__launch_bounds__(128, 4)")
-                                   : "__launch_bounds__(256, 3)";
-        std::snprintf(b, sizeof(b),
-                      "extern \"C\" __global__ void %s %s_eval_c%d(const __grid_constant__ JobTable jt) {\n"
-                      "    %s<%d, %s, %d, %s>(jt);\n}\n",
-                      lb.c_str(), pre.c_str(), c, L.body, S, def, mm, L.pol);
+        /* FP32: the deformed class of 5- and 6-dimensional sectors in phases, one block of 12 warps per SM (<= 170
+           registers, no spills); their undeformed class 128-thread blocks at 4 per SM (17 % faster than 3 on the
+           four-pole sectors of the massless double box).  FP32 below 5 dimensions: registers capped for 768 threads per
+           SM (the massive box pass is 18 % faster than with the compiler's 125 registers and 512 threads).  FP64 keeps
+           256. */
+        const bool phased = !L.f64 && qmc_gen_phased(S, c);
+        const char *lb = L.f64 ? "__launch_bounds__(256)"
+                         : phased ? "__launch_bounds__(QMC_PHASED_THREADS, 1)"
+                                  : (qmc_gen_max_block(S) == 128 ? "__launch_bounds__(128, 4)" : "__launch_bounds__(256, 3)");
+        std::snprintf(b, sizeof(b), "extern \"C\" __global__ void %s %s_eval_c%d(const __grid_constant__ JobTable jt) {\n",
+                      lb, pre.c_str(), c);
+        o += b;
+        if (phased)
+            std::snprintf(b, sizeof(b), "    eval_f32x2_phased_body<%d, %d, %s>(jt);\n}\n", S, mm, L.pol);
+        else
+            std::snprintf(b, sizeof(b), "    %s<%d, %s, %d, %s>(jt);\n}\n", L.body, S, def, mm, L.pol);
         o += b;
     }
     return o;

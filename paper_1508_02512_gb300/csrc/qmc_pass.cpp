@@ -28,6 +28,9 @@
 namespace {
 
 /* ------------------------------------------------------------------ launch planning */
+/* dynamic shared memory that a phased FP32 block may take: 227 KB less its static arrays (under 2 KB) */
+#define QMC_PHASED_SMEM (225 * 1024)
+
 /* A run: consecutive packed sectors of one class that the pass evaluates (all of the class unless the pass
    names a subset); each run becomes one job per precision and one reduction job. */
 struct Run {
@@ -264,11 +267,14 @@ int run_eval(const qmc_batch_item *items, int n, const BatchLayout &L, unsigned 
         for (size_t b0 = 0; b0 < jobs.size(); b0 += QMC_MAX_JOBS) {
             std::memset(jt.get(), 0, sizeof(JobTable));
             const size_t nj = std::min(jobs.size() - b0, (size_t)QMC_MAX_JOBS);
+            /* the phased kernel takes `grp` items of a sector at a time, one per group of k.block threads */
+            const bool phased = k.gen && k.prec == QMC_PREC_MIXED && qmc_gen_phased(k.dim, k.deform);
+            const int64_t grp = phased ? QMC_PHASED_THREADS / k.block : 1;
             int64_t total = 0;
             for (size_t q = 0; q < nj; ++q) {
                 jt->jobs[q] = jobs[b0 + q];
                 jt->jobs[q].item_begin = total;
-                total += (int64_t)jt->jobs[q].n_sect * jt->jobs[q].m * jt->jobs[q].chunks;
+                total += (int64_t)jt->jobs[q].n_sect * ((jt->jobs[q].m * jt->jobs[q].chunks + grp - 1) / grp);
             }
             jt->n_jobs = (int32_t)nj;
             jt->r = k.r;
@@ -278,8 +284,17 @@ int run_eval(const qmc_batch_item *items, int n, const BatchLayout &L, unsigned 
             if (counter >= L.n_counters) return QMC_ERR_UNSUPPORTED;
             jt->counter = counters + counter++;
             jt->smem_bytes = smem_need[k];
+            int threads = k.block;
+            if (phased) {
+                threads = QMC_PHASED_THREADS;
+                jt->block = k.block;
+                jt->state_off = jt->smem_bytes;
+                const int per_pair = qmc_phased_state(k.dim, k.maxm) * threads;
+                jt->pairs = jt->smem_bytes + 2 * per_pair <= QMC_PHASED_SMEM ? 2 : 1;
+                jt->smem_bytes += jt->pairs * per_pair;
+            }
             int per_sm = 0;
-            rc = k.gen ? qmc_gen_blocks_per_sm(k.gen, k.block, jt->smem_bytes, &per_sm)
+            rc = k.gen ? qmc_gen_blocks_per_sm(k.gen, threads, jt->smem_bytes, &per_sm)
                        : qmc_eval_blocks_per_sm(k.dim, k.deform, k.maxm, k.prec, k.block, jt->smem_bytes, &per_sm);
             if (rc) return rc;
             if (per_sm < 1) return QMC_ERR_UNSUPPORTED;
@@ -287,7 +302,7 @@ int run_eval(const qmc_batch_item *items, int n, const BatchLayout &L, unsigned 
             for (int i = 0; i < n; ++i)
                 if (items[i].pass.grid > 0) grid = std::min<int64_t>(grid, items[i].pass.grid);
             if (grid > total) grid = total;
-            rc = k.gen ? qmc_gen_launch_eval(k.gen, *jt, (int)grid, k.block, stream)
+            rc = k.gen ? qmc_gen_launch_eval(k.gen, *jt, (int)grid, threads, stream)
                        : qmc_launch_eval(k.dim, k.deform, k.maxm, k.prec, *jt, (int)grid, k.block, stream);
             if (rc) return rc;
         }
