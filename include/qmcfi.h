@@ -100,7 +100,7 @@ typedef struct {
     int32_t precision;         /* QMC_PREC_FP64 or QMC_PREC_MIXED */
     int32_t block;             /* threads per block: 0 = default (128), else 32..256 and a multiple of 32; at most
                                   128 for generated FP32 evaluators of 5- and 6-dimensional sectors */
-    int32_t points_per_thread; /* 0 = default, else 1..64 */
+    int32_t points_per_thread; /* 0 = default (16 in mixed precision, 8 in FP64, fewer for small passes), else 1..64 */
     int32_t grid;              /* blocks of the persistent kernel: 0 = one wave on the device */
     int32_t evaluator;         /* QMC_EVAL_* of the FP32 evaluation */
     int32_t reserved;

@@ -66,6 +66,32 @@ TuneKey tune_key(const PackedHeader *h, const qmc_pass *p) {
     return TuneKey{h->family, p->precision, ev, b};
 }
 
+/* Points per thread of a pass that leaves them to the library: 16 in mixed precision and 8 in FP64, less where that leaves
+   threads without points or the chip without work.
+   - The chunks of a (sector, shift) are made equally long: with n = 3001 two chunks of 12 x 128 points instead of one of
+     16 x 128 and a rest that waits for it (non-planar double box, mixed, 16 shifts: 0.584 -> 0.518 ms).
+   - Few items: half as many points below 8 items per SM (FP64 kernels run two blocks per SM, so four waves of items:
+     non-planar double box n = 1021 3.18 -> 2.43 ms in FP64, 0.339 -> 0.299 ms mixed; above the line, massless box
+     n = 8191 with 1536 items, halving costs 2 %), a quarter below one item per SM after that (massive box n = 1021,
+     FP64: 84, 59, 57 us with 8, 4, 2 points). */
+int default_points(const PackedHeader *h, const PackedSector *ps, const qmc_pass *p, int block) {
+    const bool mixed = p->precision == QMC_PREC_MIXED;
+    const int64_t SMS = 152; /* GB300 */
+    int sectors = 0;
+    for (int s = 0; s < h->n_sectors; ++s) sectors += !p->sector_active || p->sector_active[ps[s].orig_index];
+    auto chunks = [&](int P) { return (p->lattice.n + (int64_t)block * P - 1) / ((int64_t)block * P); };
+    auto items = [&](int P) { return (int64_t)sectors * p->n_shifts * chunks(P); };
+    int P = mixed ? 16 : 8;
+    const int64_t per = chunks(P) * block;
+    P = (int)((p->lattice.n + per - 1) / per);
+    if (items(P) < 8 * SMS) {
+        P = (P + 1) / 2;
+        if (items(P) < SMS) P = (P + 1) / 2;
+    }
+    if (mixed && P % 2) ++P; /* the FP32 kernels take points in pairs */
+    return P;
+}
+
 int make_plan(const PackedHeader *h, const qmc_pass *p, Plan &pl) {
     if (!h || !p) return QMC_ERR_ARG;
     if (p->lattice.n < 2 || p->lattice.n >= ((int64_t)1 << 31)) return QMC_ERR_ARG;
@@ -86,14 +112,14 @@ int make_plan(const PackedHeader *h, const qmc_pass *p, Plan &pl) {
     if (pl.block < 32 || pl.block > 256 || pl.block % 32) return QMC_ERR_ARG;
     if (p->precision == QMC_PREC_MIXED && p->evaluator != QMC_EVAL_TABLE && pl.block > qmc_gen_max_block(h->dim))
         return QMC_ERR_ARG;
-    pl.P = P ? P : (p->precision == QMC_PREC_MIXED ? 16 : 8);
+    const PackedSector *ps =
+        reinterpret_cast<const PackedSector *>(reinterpret_cast<const unsigned char *>(h) + h->sectors_off);
+    pl.P = P ? P : default_points(h, ps, p, pl.block);
     if (pl.P < 1 || pl.P > 64) return QMC_ERR_ARG;
     for (int j = 0; j < h->dim; ++j)
         if (p->lattice.z[j] == 0 || (int64_t)p->lattice.z[j] >= p->lattice.n) return QMC_ERR_ARG;
     const int64_t C = (int64_t)pl.block * pl.P;
     pl.chunks = (p->lattice.n + C - 1) / C;
-    const PackedSector *ps =
-        reinterpret_cast<const PackedSector *>(reinterpret_cast<const unsigned char *>(h) + h->sectors_off);
     int64_t off = 0;
     pl.runs.clear();
     for (int c = 0; c < QMC_N_CLASSES; ++c) {
