@@ -605,9 +605,27 @@ Cache &cache() {
 
 const Lang &lang_of(int precision) { return precision == QMC_PREC_FP64 ? kF64 : kF32; }
 
-/* cache key: the family and the precision of the generated evaluator */
+/* Cache key: the family and the precision of the generated evaluator.  Every pass looks its kernels up, so the family is
+   taken from the header (qmc_prepare hashed the exponents of all terms into it; hashing them again took 0.5 ms per
+   look-up for a two-loop image, several times per pass), together with what the generated code depends on besides
+   the exponents, in case the image was saved by a library whose family did not cover it. */
 uint64_t module_key(const PackedHeader *h, int precision) {
-    return family_key(h) ^ (precision == QMC_PREC_FP64 ? 0x9E3779B97F4A7C15ull : 0ull);
+    Fnv f;
+    f.add_i(QMC_JIT_GENERATOR_VERSION);
+    f.add_i((int64_t)h->family);
+    f.add_i(h->dim);
+    f.add_i(h->n_sectors);
+    f.add_i(h->n_terms_total);
+    f.add_i(h->eU0);
+    f.add_i(h->eU1);
+    f.add_i(h->eF0);
+    f.add_i(h->eF1);
+    for (int c = 0; c < QMC_N_CLASSES; ++c) {
+        f.add_i(h->class_begin[c]);
+        f.add_i(h->class_end[c]);
+        f.add_i(maxm_of(h, c));
+    }
+    return f.v ^ (precision == QMC_PREC_FP64 ? 0x9E3779B97F4A7C15ull : 0ull);
 }
 
 /* compile and load (no lock held) */
