@@ -1868,7 +1868,6 @@ struct c2 {
 DEV c2 mkc2(float2 re, float2 im) { return c2{re, im}; }
 DEV c2 zero_c2() { return c2{bc2(0.f), bc2(0.f)}; }
 DEV c2 cadd2(c2 a, c2 b) { return c2{add2(a.re, b.re), add2(a.im, b.im)}; }
-DEV c2 csub2(c2 a, c2 b) { return c2{sub2(a.re, b.re), sub2(a.im, b.im)}; }
 DEV c2 cscale2(c2 a, float2 s) { return c2{mul2(a.re, s), mul2(a.im, s)}; }
 /* as cmulf per lane: (fma(a.re, b.re, rn(-a.im b.im)), fma(a.re, b.im, rn(a.im b.re))) */
 DEV c2 cmul2(c2 a, c2 b) { return c2{fma2(a.re, b.re, neg2(mul2(a.im, b.im))), fma2(a.re, b.im, mul2(a.im, b.re))}; }
