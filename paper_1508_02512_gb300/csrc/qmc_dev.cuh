@@ -15,8 +15,8 @@
  *   (compensated), so results do not depend on which block ran which item (Eqs. 16 and 18).
  * qmc_points_kernel: the same per-point device code on explicit lattice indices (sampled checks).
  *
- * The path is bound by FP64 arithmetic (no dense contraction, nothing streamed from HBM), so no tensor cores
- * or TMA are used: tables live in shared memory, points are generated, outputs are a few KB.
+ * The FP64 path is bound by the FP64 pipe, the FP32 path by instruction issue and the FP32 pipe's operand ports (no dense
+ * contraction, nothing streamed from HBM), so no tensor cores or TMA are used: tables live in shared memory, points are generated, outputs are a few KB.
  *
  * This header holds device code only, so that it also compiles at run time (NVRTC) together with the
  * polynomial code generated for one family of sector tables; the host launchers are in qmc_device.cuh.

@@ -10,7 +10,8 @@
  * every sector's monomials as straight-line CUDA: each distinct monomial is formed once, as its parent
  * monomial times one variable (the parent drops one power of the highest-index variable, so the factors are
  * multiplied in the same order as in the table evaluator), and every term adds coefficient x monomial to its
- * polynomial with the same two FMAs (coefficient hi + lo) as the table evaluator.  Coefficients are still read
+ * polynomial with the same two FMAs (coefficient hi + lo) as the table evaluator; the FP64 polynomials of deformed
+ * sectors are nested instead (emit_horner).  Coefficients are still read
  * from the sector's staged term table, so a new kinematic point of the same family reuses the compiled code.
  *
  * The generated source includes the kernel templates of qmc_dev.cuh (embedded into this library at build

@@ -74,11 +74,10 @@ TuneKey tune_key(const PackedHeader *h, const qmc_pass *p) {
      non-planar double box n = 1021 3.18 -> 2.43 ms in FP64, 0.339 -> 0.299 ms mixed; above the line, massless box
      n = 8191 with 1536 items, halving costs 2 %), a quarter below one item per SM after that (massive box n = 1021,
      FP64: 84, 59, 57 us with 8, 4, 2 points). */
-int default_points(const PackedHeader *h, const PackedSector *ps, const qmc_pass *p, int block) {
+int default_points(const PackedHeader *h, const qmc_pass *p, int block) {
     const bool mixed = p->precision == QMC_PREC_MIXED;
     const int64_t SMS = 152; /* GB300 */
-    int sectors = 0;
-    for (int s = 0; s < h->n_sectors; ++s) sectors += !p->sector_active || p->sector_active[ps[s].orig_index];
+    const int sectors = h->n_sectors; /* also where only some are active: their sums are those of the whole pass */
     auto chunks = [&](int P) { return (p->lattice.n + (int64_t)block * P - 1) / ((int64_t)block * P); };
     auto items = [&](int P) { return (int64_t)sectors * p->n_shifts * chunks(P); };
     int P = mixed ? 16 : 8;
@@ -112,14 +111,14 @@ int make_plan(const PackedHeader *h, const qmc_pass *p, Plan &pl) {
     if (pl.block < 32 || pl.block > 256 || pl.block % 32) return QMC_ERR_ARG;
     if (p->precision == QMC_PREC_MIXED && p->evaluator != QMC_EVAL_TABLE && pl.block > qmc_gen_max_block(h->dim))
         return QMC_ERR_ARG;
-    const PackedSector *ps =
-        reinterpret_cast<const PackedSector *>(reinterpret_cast<const unsigned char *>(h) + h->sectors_off);
-    pl.P = P ? P : default_points(h, ps, p, pl.block);
+    pl.P = P ? P : default_points(h, p, pl.block);
     if (pl.P < 1 || pl.P > 64) return QMC_ERR_ARG;
     for (int j = 0; j < h->dim; ++j)
         if (p->lattice.z[j] == 0 || (int64_t)p->lattice.z[j] >= p->lattice.n) return QMC_ERR_ARG;
     const int64_t C = (int64_t)pl.block * pl.P;
     pl.chunks = (p->lattice.n + C - 1) / C;
+    const PackedSector *ps =
+        reinterpret_cast<const PackedSector *>(reinterpret_cast<const unsigned char *>(h) + h->sectors_off);
     int64_t off = 0;
     pl.runs.clear();
     for (int c = 0; c < QMC_N_CLASSES; ++c) {
