@@ -70,7 +70,7 @@ TuneKey tune_key(const PackedHeader *h, const qmc_pass *p) {
    threads without points or the chip without work.
    - The chunks of a (sector, shift) are made equally long: with n = 3001 two chunks of 12 x 128 points instead of one of
      16 x 128 and a rest that waits for it (non-planar double box, mixed, 16 shifts: 0.584 -> 0.518 ms).
-   - Few items: half as many points below 8 items per SM (FP64 kernels run two blocks per SM, so four waves of items:
+   - Few items: half as many points below 6 items per SM (FP64 kernels run two blocks per SM, so three waves of items:
      non-planar double box n = 1021 3.18 -> 2.43 ms in FP64, 0.339 -> 0.299 ms mixed; above the line, massless box
      n = 8191 with 1536 items, halving costs 2 %), a quarter below one item per SM after that (massive box n = 1021,
      FP64: 84, 59, 57 us with 8, 4, 2 points). */
@@ -83,7 +83,7 @@ int default_points(const PackedHeader *h, const qmc_pass *p, int block) {
     int P = mixed ? 16 : 8;
     const int64_t per = chunks(P) * block;
     P = (int)((p->lattice.n + per - 1) / per);
-    if (items(P) < 8 * SMS) {
+    if (items(P) < 6 * SMS) {
         P = (P + 1) / 2;
         if (items(P) < SMS) P = (P + 1) / 2;
     }

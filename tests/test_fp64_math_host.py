@@ -127,7 +127,7 @@ def test_determinant_with_and_without_zeroed_coordinates(lib, S):
 
 def test_default_points_per_thread():
     """Passes that leave the launch shape open take the scratch of the shape they stand for: equal chunks, half the points
-    below 8 items per SM (152), a quarter below one after that, an even number in mixed precision."""
+    below 6 items per SM (152), a quarter below one after that, an even number in mixed precision."""
     cfg = W.CONFIG3
     prep = api.prepare(T.compile_integral(cfg.topology, T.zero_invariants_of(cfg.topology, cfg.point)), cfg.kin,
                        cfg.order_min, cfg.order_max)
