@@ -230,21 +230,23 @@ void emit_horner(std::string &o, const PolySet &P, int acc, std::vector<HTerm> t
     const std::string ind(4 + 2 * depth, ' ');
     const std::string a = "a" + std::to_string(acc), v = P.complex_ ? "z[" : "t[";
     bool have = false; /* the accumulator holds a value */
-    for (size_t k = 0; k < terms.size(); ++k) {
+    /* the constants: one as a rule, several where a table lists a monomial more than once (their coefficients add up) */
+    std::vector<HTerm> rest;
+    for (const HTerm &t : terms) {
         bool constant = true;
-        for (int j = 0; j < P.S; ++j) constant = constant && terms[k].e[j] == 0;
-        if (!constant) continue;
-        if (terms[k].dead) {
-            terms.erase(terms.begin() + k);
-            break;
+        for (int j = 0; j < P.S; ++j) constant = constant && t.e[j] == 0;
+        if (!constant) {
+            rest.push_back(t);
+            continue;
         }
-        const std::string c = "C[" + std::to_string(terms[k].term) + "].c";
-        o += ind + a + (P.complex_ ? ".x" : "") + " = " + c + ";\n";
-        if (P.complex_) o += ind + a + ".y = 0;\n";
-        terms.erase(terms.begin() + k);
+        if (t.dead) continue;
+        const std::string c = "C[" + std::to_string(t.term) + "].c";
+        o += ind + a + (P.complex_ ? ".x" : "") + (have ? " += " : " = ") + c + ";\n";
+        if (P.complex_ && !have) o += ind + a + ".y = 0;\n";
         have = true;
-        break;
     }
+    terms.swap(rest);
+    /* every term left holds a variable, so each step takes at least one away */
     while (!terms.empty()) {
         int best = 0, most = -1;
         for (int j = 0; j < P.S; ++j) {
