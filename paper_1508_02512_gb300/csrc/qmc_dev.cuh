@@ -117,7 +117,8 @@ DEV double qlog(double x) {
     return fma(e, LN2, qmc_logtab.log_c[k]) + fma(e, LN2_LO, p);
 }
 
-/* principal log */ /* of U and of the q_j takes its argument from qatan2; log(F - i0) has a negative real F at -pi */
+/* principal log */
+/* its imaginary part is qatan2 for U and the q_j; for F - i0 a negative real F lies at -pi */
 DEV double arg_mi0(cd z) { return z.y == 0.0 ? (z.x < 0.0 ? -QMC_PI : 0.0) : qatan2(z.y, z.x); }
 
 /* ------------------------------------------------------------------ periodising transform (Eq. 21, order r) */
@@ -423,6 +424,30 @@ struct EnableIf<true> {
 };
 
 
+/* Exponents of FP64 numbers, on the integer pipes */
+DEV unsigned biased_exp(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7FFu; }
+/* bound on |log2 x|, x > 0; above 1000 for zero, subnormals, infinities and NaN */
+DEV int exp_size(double x) {
+    const int e = (int)biased_exp(x) - 1023;
+    return (e < 0 ? -e : e) + 1;
+}
+/* v^e to the product num / dnm times 2^e2, by v's mantissa in [1, 2) and exponent (zero, infinity and NaN as they are) */
+DEV void mul_mantissa(double &num, double &dnm, int &e2, double v, int e) {
+    if (biased_exp(v) == 0) {
+        v *= 18014398509481984.0; /* 2^54: subnormal numbers become normal */
+        e2 -= 54 * e;
+    }
+    const int be = (int)biased_exp(v);
+    if (be > 0 && be < 2047) {
+        e2 += (be - 1023) * e;
+        v = __longlong_as_double((__double_as_longlong(v) & 0x000FFFFFFFFFFFFFLL) | 0x3FF0000000000000LL);
+    }
+    for (int k = 0; k < e; ++k) num *= v;
+    for (int k = 0; k > e; --k) dnm *= v;
+}
+/* largest exponent of a product of moduli that shares one reciprocal: what it multiplies stays 2^100 from overflowing early */
+#define QMC_SHARED_DEN_EXP 200
+
 /* G at the point tt (t with the subset Y zeroed): returns its eps^0 value G0 and, with needX, the eps-coefficient X of
    its logarithm, so that G(eps) = G0 exp(X eps) (Sec. II, Eq. 9 with the deformation of Eq. 14).  First the undeformed
    class, where everything is real. */
@@ -487,8 +512,17 @@ DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *t
         const cd iU = mk(U.x * f, -U.y * f);
         G = cmul(G, cpow_inv(iU, iU, -ex.eU0));
     }
-    /* prod_j (t_j q_j)^{A_j}, t_j only for A_j >= 0: a product with q_j is two FMAs, and 1/q_j = (1 + i d_j)/(1 + d_j^2) */
+    /* prod_j (t_j q_j)^{A_j}, t_j only for A_j >= 0: a product with q_j is two FMAs, and 1/q_j = (1 + i d_j)/(1 + d_j^2).
+       The moduli 1 + d_j^2 share one reciprocal while their product is moderate.  d_j carries the scale of the kinematics
+       (F~ is not normalised), so before lambda has been halved far enough it can be anything: then the factors are
+       divided out one by one. */
     double re = s.D, den = 1.0;
+    if (s.sigma > 0) {
+#pragma unroll
+        for (int j = 0; j < S; ++j)
+            for (int k = 0; k > s.A[j]; --k) den *= fma(d[j], d[j], 1.0);
+    }
+    const bool shared_den = biased_exp(den) < 1023u + QMC_SHARED_DEN_EXP; /* den >= 1; false for infinities and NaN */
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         for (int k = 0; k < s.A[j]; ++k) {
@@ -496,21 +530,30 @@ DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *t
             G = mk(fma(G.y, d[j], G.x), fma(-G.x, d[j], G.y));
         }
         for (int k = 0; k > s.A[j]; --k) {
-            den *= fma(d[j], d[j], 1.0);
-            G = mk(fma(-G.y, d[j], G.x), fma(G.x, d[j], G.y));
+            if (shared_den) {
+                G = mk(fma(-G.y, d[j], G.x), fma(G.x, d[j], G.y));
+            } else {
+                const double f = __drcp_rn(fma(d[j], d[j], 1.0));
+                G = cmul(G, mk(f, d[j] * f));
+            }
         }
     }
-    if (s.sigma > 0) re *= qrcp(den);
+    if (s.sigma > 0 && shared_den) re *= qrcp(den);
     G0 = cscale(G, re);
     X = mk(0.0, 0.0);
     if (needX) {
         /* eU1 log U - eF1 log F + sum_j B_j log q_j (and B_j log t_j where A_j != -1).  The moduli of U and of the q_j
-           share one logarithm: U and q_j do not scale with the kinematics, so their powers stay in range. */
+           share one logarithm, of num / dnm.  Both are products of up to |eU1| + sum |B_j| factors that grow with the
+           kinematics (U through z), so their exponents are added up first (integers, off the FP64 pipe); where they
+           could leave the normal range the mantissas are multiplied and the exponents join as a multiple of ln 2.
+           Without and with the
+           check, 16 shifts: non-planar double box n = 16381 34.26, 34.34 ms; massive box n = 262139 4.79, 4.76 ms. */
         const double U2 = fma(U.x, U.x, U.y * U.y);
         double num = 1.0, dnm = 1.0, xr = 0.0;
         double xi = (double)ex.eU1 * qatan2(U.y, U.x);
         for (int k = 0; k < ex.eU1; ++k) num *= U2;
         for (int k = 0; k > ex.eU1; --k) dnm *= U2;
+        int range = abs(ex.eU1) * exp_size(U2);
 #pragma unroll
         for (int j = 0; j < S; ++j) {
             if (s.B[j] != 0) {
@@ -518,11 +561,21 @@ DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *t
                 const double q2 = fma(d[j], d[j], 1.0);
                 for (int k = 0; k < s.B[j]; ++k) num *= q2;
                 for (int k = 0; k > s.B[j]; --k) dnm *= q2;
+                range += abs(s.B[j]) * exp_size(q2);
                 xi = fma(-qmc_sec.B[j], qatan2(d[j], 1.0), xi);
             }
         }
+        int e2 = 0;
+        if (range > 1000) {
+            num = dnm = 1.0;
+            mul_mantissa(num, dnm, e2, U2, ex.eU1);
+#pragma unroll
+            for (int j = 0; j < S; ++j) mul_mantissa(num, dnm, e2, fma(d[j], d[j], 1.0), s.B[j]);
+        }
         const double eF1 = (double)ex.eF1;
-        X.x = fma(0.5, fma(-eF1, qlog(F2), qlog(num * qrcp(dnm))), xr);
+        double l = qlog(num * qrcp(dnm));
+        if (e2 != 0) l = fma((double)e2, 0.6931471805599453, l);
+        X.x = fma(0.5, fma(-eF1, qlog(F2), l), xr);
         X.y = fma(-eF1, arg_mi0(F), xi);
     }
 }
