@@ -193,9 +193,9 @@ int qmc_launch_probe(int dim, int deform, int maxm, const ProbeArgs &a, void *st
 
 /* Generated evaluators (qmc_jit.cpp): the evaluation kernel (QMC_PREC_FP64 or _MIXED = FP32) of a family's
    module for sector class cls
-   (compiled and loaded on first use), its occupancy and launch.  Kernel handles are cudaKernel_t values passed
-   as const void *. */
-int qmc_gen_kernel(const void *packed_host, int precision, int cls, const void **eval_kernel);
+   (compiled and loaded on first use), its occupancy and launch.  family: qmc_family_key of the image.  Kernel handles are
+   cudaKernel_t values passed as const void *. */
+int qmc_gen_kernel(const void *packed_host, uint64_t family, int precision, int cls, const void **eval_kernel);
 uint64_t qmc_family_key(const void *packed_host); /* computed from the image, not read from its header */
 int qmc_gen_max_block(int dim);                  /* largest block of a generated kernel for sectors of this dimension */
 /* Whether the generated FP32 kernel of this class works in phases (eval_f32x2_phased_body): then it runs

@@ -211,7 +211,7 @@ struct LaunchKey {
 
 bool use_generated(const qmc_pass &p) { return p.precision == QMC_PREC_MIXED && p.evaluator != QMC_EVAL_TABLE; }
 /* FP64 jobs: generated unless the pass asks for the table */
-bool use_generated64(const qmc_pass &p, const PackedHeader *) { return p.evaluator != QMC_EVAL_TABLE; }
+bool use_generated64(const qmc_pass &p) { return p.evaluator != QMC_EVAL_TABLE; }
 
 /* Evaluation launches of a batch: every (pass, class, precision) becomes a job; jobs sharing a kernel
    instantiation and launch shape go into one persistent launch (tables of up to QMC_MAX_JOBS jobs). */
@@ -225,11 +225,17 @@ int run_eval(const qmc_batch_item *items, int n, const BatchLayout &L, unsigned 
     if (rc) return rc;
     std::map<LaunchKey, std::vector<Job>> groups;
     std::map<LaunchKey, int> smem_need;
+    const void *family_of = nullptr;
+    uint64_t family = 0;
     for (int i = 0; i < n; ++i) {
         const qmc_batch_item &b = items[i];
         const PackedHeader *h = header_of(b.packed_host);
         const Plan &pl = L.plans[i];
         const bool mixed = b.pass.precision == QMC_PREC_MIXED;
+        if (use_generated64(b.pass) && b.packed_host != family_of) { /* the passes of an integral follow one another */
+            family = qmc_family_key(b.packed_host);
+            family_of = b.packed_host;
+        }
         for (const Run &run : pl.runs) {
             const int c = run.cls;
             for (int prec = 0; prec < 2; ++prec) {
@@ -266,10 +272,10 @@ int run_eval(const qmc_batch_item *items, int n, const BatchLayout &L, unsigned 
                 J.eF1 = h->eF1;
                 const void *gen = nullptr;
                 if (prec == 1 && use_generated(b.pass)) {
-                    rc = qmc_gen_kernel(b.packed_host, QMC_PREC_MIXED, c, &gen);
+                    rc = qmc_gen_kernel(b.packed_host, family, QMC_PREC_MIXED, c, &gen);
                     if (rc) return rc;
-                } else if (prec == 0 && !fp64_only && use_generated64(b.pass, h)) {
-                    rc = qmc_gen_kernel(b.packed_host, QMC_PREC_FP64, c, &gen);
+                } else if (prec == 0 && !fp64_only && use_generated64(b.pass)) {
+                    rc = qmc_gen_kernel(b.packed_host, family, QMC_PREC_FP64, c, &gen);
                     if (rc) return rc;
                 }
                 const LaunchKey key{h->dim, c, class_maxm(h, c), prec == 0 ? QMC_PREC_FP64 : QMC_PREC_MIXED, pl.block,
