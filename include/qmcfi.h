@@ -100,7 +100,9 @@ typedef struct {
     int32_t precision;         /* QMC_PREC_FP64 or QMC_PREC_MIXED */
     int32_t block;             /* threads per block: 0 = default (128), else 32..256 and a multiple of 32; at most
                                   128 for generated FP32 evaluators of 5- and 6-dimensional sectors */
-    int32_t points_per_thread; /* 0 = default (16 in mixed precision, 8 in FP64, fewer for small passes), else 1..64 */
+    int32_t points_per_thread; /* 1..64, or 0: the library's choice, which depends on precision, block, lattice.n, n_shifts
+                                  and the number of sectors of the image (not on sector_active): 16 in mixed precision, 8
+                                  in FP64, fewer for small passes, or the autotuned number */
     int32_t grid;              /* blocks of the persistent kernel: 0 = one wave on the device */
     int32_t evaluator;         /* QMC_EVAL_* of the FP32 evaluation */
     int32_t reserved;
@@ -172,7 +174,9 @@ size_t qmc_scratch_bytes(const void *packed, const qmc_pass *pass);
  * [0,1).  lambda_dev: one deformation parameter per sector (table order).  scratch_dev: at least
  * qmc_scratch_bytes() bytes, 256-byte aligned, owned by the caller; contents need no initialisation and are
  * overwritten.  Sums are deterministic: independent of grid size and scheduling for fixed block and
- * points_per_thread.  Errors: QMC_ERR_ARG, QMC_ERR_UNSUPPORTED, QMC_ERR_MEMORY (scratch too small), QMC_ERR_CUDA.
+ * points_per_thread.  With both given, the sums of a shift do not depend on the other shifts of the pass either (shifts may
+ * be shared out over passes or processes without changing a bit); with points_per_thread = 0 their last bits can differ
+ * between passes of different n_shifts.  Errors: QMC_ERR_ARG, QMC_ERR_UNSUPPORTED, QMC_ERR_MEMORY (scratch too small), QMC_ERR_CUDA.
  */
 int qmc_eval_sums(const void *packed_host, const void *packed_dev, const qmc_pass *pass, const double *shifts_dev,
                   const double *lambda_dev, void *scratch_dev, size_t scratch_bytes, double *sums_dev,

@@ -70,13 +70,24 @@ TuneKey tune_key(const PackedHeader *h, const qmc_pass *p) {
    threads without points or the chip without work.
    - The chunks of a (sector, shift) are made equally long: with n = 3001 two chunks of 12 x 128 points instead of one of
      16 x 128 and a rest that waits for it (non-planar double box, mixed, 16 shifts: 0.584 -> 0.518 ms).
-   - Few items: half as many points below 6 items per SM (FP64 kernels run two blocks per SM, so three waves of items:
-     non-planar double box n = 1021 3.18 -> 2.43 ms in FP64, 0.339 -> 0.299 ms mixed; above the line, massless box
-     n = 8191 with 1536 items, halving costs 2 %), a quarter below one item per SM after that (massive box n = 1021,
-     FP64: 84, 59, 57 us with 8, 4, 2 points). */
+   - Few items: half as many points below 6 items per SM.  Four FP64 blocks share an SM, so that is one and a half waves,
+     and sectors of different cost leave some SMs idle at its end.  The more the sectors differ the higher the line could
+     be; it lies between the families (n = 1021 in FP64 and 2039 mixed, full against half the points):
+                                 at 5 items per SM       at 7                    at 10
+       non-planar double box     3127, 2312 us FP64      3425, 3141              4520, 4451
+                                 389, 274 mixed          404, 379                500, 499
+       four-pole double box      1382, 1006 (at 4.7)     1473, 1211 (at 6.6)     1903, 1653
+                                 293, 229                339, 268                428, 330
+       massless box              436, 408                606, 552                747, 768
+                                 67, 73                  89, 87                  115, 115
+       massive box               241, 251                327, 344                462, 487
+                                 44, 48                  54, 56                  68, 72
+   - A quarter where half the points still leave less than one item per SM (non-planar double box, 2 shifts: 1200, 615,
+     496 us with 8, 4, 2 points; massive box, 19 shifts: 68, 45, 44).
+   The number of SMs is the GB300's and not the device's: the sums' last bits depend on the shape, and so not on the part. */
 int default_points(const PackedHeader *h, const qmc_pass *p, int block) {
     const bool mixed = p->precision == QMC_PREC_MIXED;
-    const int64_t SMS = 152; /* GB300 */
+    const int64_t SMS = 152;
     const int sectors = h->n_sectors; /* also where only some are active: their sums are those of the whole pass */
     auto chunks = [&](int P) { return (p->lattice.n + (int64_t)block * P - 1) / ((int64_t)block * P); };
     auto items = [&](int P) { return (int64_t)sectors * p->n_shifts * chunks(P); };
