@@ -226,7 +226,8 @@ DEV double rcp_seed(double x) {
     return r;
 }
 /* 1/x from an approximation r good to some 20 bits, by one step of Householder's third-order iteration: with
-   e = 1 - x r, 1/x = r (1 + e + e^2 + ...) and the first term left out is e^3 < 2^-57.  Three FMAs; the correctly
+   e = 1 - x r, 1/x = r (1 + e + e^2 + ...) and the first term left out is e^3 < 2^-57, so
+   the result is within 0.51 units in the last place (0.508 found over 2e6 arguments).  Three FMAs; the correctly
    rounded __drcp_rn takes as much of the FP64 pipe as 5.3 of them (measured), and is left for arguments whose
    reciprocal could leave the normal range. */
 DEV double qrcp(double x) {
@@ -655,7 +656,8 @@ DEV void subset_factor(double (&V)[MAXM + 1], int z, const double *a, bool inY, 
    Bound by the FP64 pipe.  With the series and their products hoisted out of the subset loop, no arithmetic on zero
    imaginary parts or zero coefficients, and no logarithm where the order does not ask for it, the FP64 passes (16
    shifts) went from 32.2 to 16.2 ms (four-pole double box, n = 8191) and, with 8 shifts, from 5.36 to 2.88 ms (massless
-   box, n = 65521), with the same point values bit for bit. */
+   box, n = 65521).  The sum over the subsets rounds as it did with every step in the loop; the weight, one product of all
+   x (1 - x) (weight64), in its last digit otherwise. */
 template <int S, bool DEF, int MAXM, class Pol>
 DEV typename EnableIf<!DEF>::type point_integrand(const PackedSector &s, const Pol &P, const double *x, int r, double,
                                                   const Exps &ex, cd (&out)[MAXM + 1], uint32_t &) {

@@ -20,8 +20,10 @@ inline const PackedSector *sectors_of(const void *packed) {
 }
 inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? QMC_OK : QMC_ERR_CUDA; }
 
-/* cost of an FP64 evaluation per algorithmic flop relative to FP32 (the generated kernels' measured rates differ by
-   20-33x): for the choice of each sector's precision, and for charging a serving round's time to its requests */
+/* cost of an FP64 evaluation per algorithmic flop relative to FP32, for the choice of each sector's precision (part of
+   what qmcfi.h says of qmc_choose_precision) and for charging a serving round's time to its requests.  The generated
+   kernels' rates differ by 21 (non-planar double box: 7.83e9 and 3.67e8 evaluations per second), 22 (massive box) and 13
+   (four-pole double box), so 30 leans towards FP32 and islands; another value would move sectors to another precision. */
 #define QMC_FP64_COST 30.0
 
 namespace qmci {

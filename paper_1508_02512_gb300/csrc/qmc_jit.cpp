@@ -74,11 +74,13 @@ struct Fnv {
 };
 
 /* The family: a hash of the header's and the sectors' structure and of every term's exponents, read from the image itself,
-   so that an image gets the code of its own terms whatever its header says.  Every pass takes it once per image: four
-   chains of word-wise products keep the multiplier busy (two-loop image, 15404 terms: 12 us against 119 us for
-   one byte-wise chain). */
+   so that an image gets the code of its own terms whatever its header says.  Every pass takes it once per image.  A chain
+   of word-wise products waits for each product, so eight chains run side by side: 4.6 us for the 15404 terms of a two-loop
+   image in cache and 14 us from memory (four chains 5.7 and 14, one byte-wise chain 119). */
 uint64_t family_key(const PackedHeader *h) {
-    uint64_t v[4] = {0x9E3779B97F4A7C15ull, 0xC2B2AE3D27D4EB4Full, 0x165667B19E3779F9ull, 0xD6E8FEB86659FD93ull};
+    constexpr int CHAINS = 8;
+    uint64_t v[CHAINS];
+    for (int i = 0; i < CHAINS; ++i) v[i] = 0x9E3779B97F4A7C15ull * (i + 1);
     auto mix = [](uint64_t a, uint64_t w) {
         a = (a ^ w) * 0xFF51AFD7ED558CCDull; /* odd: one step loses nothing of the word */
         return a ^ (a >> 32);
@@ -108,13 +110,19 @@ uint64_t family_key(const PackedHeader *h) {
         for (int16_t g : p.gstart) add(g);
         for (int16_t g : p.hstart) add(g);
         const PackedTermF *t = tf + p.term0;
-        for (int k = 0; k < p.n_terms; ++k) {
+        auto exps = [t](int k) {
             uint64_t e;
             std::memcpy(&e, t[k].e, 8);
-            v[k & 3] = mix(v[k & 3], e);
-        }
+            return e;
+        };
+        int k = 0;
+        for (; k + CHAINS <= p.n_terms; k += CHAINS)
+            for (int i = 0; i < CHAINS; ++i) v[i] = mix(v[i], exps(k + i));
+        for (; k < p.n_terms; ++k) v[0] = mix(v[0], exps(k));
     }
-    return mix(mix(mix(v[0], v[1]), v[2]), v[3]);
+    uint64_t f = v[0];
+    for (int i = 1; i < CHAINS; ++i) f = mix(f, v[i]);
+    return f;
 }
 
 /* ---------------------------------------------------------------- code generation */
@@ -520,11 +528,13 @@ std::string generate(const PackedHeader *h, const Lang &L) {
         if (h->class_end[c] <= h->class_begin[c]) continue;
         const char *def = c == 1 ? "true" : "false";
         const int mm = maxm_of(h, c);
-        /* FP32: the deformed class of 5- and 6-dimensional sectors in phases, one block of 12 warps per SM (<= 170
-           registers, no spills); their undeformed class 128-thread blocks at 4 per SM (17 % faster than 3 on the
-           four-pole sectors of the massless double box).  FP32 below 5 dimensions: registers capped for 768 threads per
-           SM (the massive box pass is 18 % faster than with the compiler's 125 registers and 512 threads).  FP64 keeps
-           256. */
+        /* FP32: the deformed class of 5- and 6-dimensional sectors in phases, one block of 16 warps per SM: 128
+           registers, and in the two-loop families 252 bytes of spill stores and 320 of loads per thread; 12 warps at up to
+           168 registers are 0 to 9 % slower (eval_f32x2_phased_body).  Their undeformed class 128-thread blocks at 4 per SM
+           (17 % faster than 3 on the four-pole sectors of the massless double box).  FP32 below 5 dimensions: registers
+           capped for 768 threads per SM (the massive box pass is 18 % faster than with the compiler's 125 registers and
+           512 threads).  FP64: blocks of up to 256 threads; the compiler takes 114 to 128 registers, so four of the default
+           128 threads share an SM. */
         const bool phased = !L.f64 && qmc_gen_phased(S, c);
         const char *lb = L.f64 ? "__launch_bounds__(256)"
                          : phased ? "__launch_bounds__(QMC_PHASED_THREADS, 1)"
