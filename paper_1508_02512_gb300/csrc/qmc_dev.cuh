@@ -425,29 +425,58 @@ struct EnableIf<true> {
 };
 
 
-/* Exponents of FP64 numbers, on the integer pipes */
-DEV unsigned biased_exp(double x) { return ((unsigned)__double2hiint(x) >> 20) & 0x7FFu; }
-/* bound on |log2 x|, x > 0; above 1000 for zero, subnormals, infinities and NaN */
-DEV int exp_size(double x) {
-    const int e = (int)biased_exp(x) - 1023;
-    return (e < 0 ? -e : e) + 1;
+/* Products over the q_j = 1 - i d_j of a deformed point, where they could leave the range of a double.  d_j carries the
+   scale of the kinematics (F~ is not normalised): before lambda has been halved far enough it can be anything.  The usual
+   case is inlined in eval_G; these are functions of their own, because the compiler would execute both sides of a short
+   branch, and the FP64 pipe is the bound (non-planar double box, n = 1021, one shift: 303 us without them, 318-323 with
+   both forms inlined, 304 as they are). */
+DEV int exponent(double x) { return (int)(((unsigned)__double2hiint(x) >> 20) & 0x7FFu) - 1023; } /* 1024: infinity, NaN */
+/* bound on log2(1 + d^2), on the integer pipes */
+DEV int modulus_exponent(double d) {
+    const int e = exponent(d);
+    return e < 0 ? 1 : 2 * e + 3;
 }
-/* v^e to the product num / dnm times 2^e2, by v's mantissa in [1, 2) and exponent (zero, infinity and NaN as they are) */
-DEV void mul_mantissa(double &num, double &dnm, int &e2, double v, int e) {
-    if (biased_exp(v) == 0) {
-        v *= 18014398509481984.0; /* 2^54: subnormal numbers become normal */
-        e2 -= 54 * e;
+template <int S>
+struct Contour {
+    double d[S];
+};
+/* G prod_j q_j^{A_j}, factor by factor */
+template <int S>
+__device__ __noinline__ cd times_q(const PackedSector &s, Contour<S> c, cd G) {
+#pragma unroll
+    for (int j = 0; j < S; ++j) {
+        for (int k = 0; k < s.A[j]; ++k) G = cmul(G, mk(1.0, -c.d[j]));
+        for (int k = 0; k > s.A[j]; --k) {
+            const double f = __drcp_rn(fma(c.d[j], c.d[j], 1.0));
+            G = cmul(G, mk(f, c.d[j] * f));
+        }
     }
-    const int be = (int)biased_exp(v);
-    if (be > 0 && be < 2047) {
-        e2 += (be - 1023) * e;
+    return G;
+}
+/* v^k to the product num / dnm: its mantissa in [1, 2), and its exponent to e2 (zero, infinity and NaN as they are) */
+DEV void mul_mantissa(double &num, double &dnm, int &e2, double v, int k) {
+    if (exponent(v) == -1023) {
+        v *= 18014398509481984.0; /* 2^54: subnormal numbers become normal */
+        e2 -= 54 * k;
+    }
+    const int e = exponent(v);
+    if (e > -1023 && e < 1024) {
+        e2 += e * k;
         v = __longlong_as_double((__double_as_longlong(v) & 0x000FFFFFFFFFFFFFLL) | 0x3FF0000000000000LL);
     }
-    for (int k = 0; k < e; ++k) num *= v;
-    for (int k = 0; k > e; --k) dnm *= v;
+    for (int i = 0; i < k; ++i) num *= v;
+    for (int i = 0; i > k; --i) dnm *= v;
 }
-/* largest exponent of a product of moduli that shares one reciprocal: what it multiplies stays 2^100 from overflowing early */
-#define QMC_SHARED_DEN_EXP 200
+/* eU1 log U2 + sum_j B_j log(1 + d_j^2) */
+template <int S>
+__device__ __noinline__ double log_moduli(const PackedSector &s, Contour<S> c, double U2, int eU1) {
+    double num = 1.0, dnm = 1.0;
+    int e2 = 0;
+    mul_mantissa(num, dnm, e2, U2, eU1);
+#pragma unroll
+    for (int j = 0; j < S; ++j) mul_mantissa(num, dnm, e2, fma(c.d[j], c.d[j], 1.0), s.B[j]);
+    return fma((double)e2, 0.6931471805599453, qlog(num * qrcp(dnm)));
+}
 
 /* G at the point tt (t with the subset Y zeroed): returns its eps^0 value G0 and, with needX, the eps-coefficient X of
    its logarithm, so that G(eps) = G0 exp(X eps) (Sec. II, Eq. 9 with the deformation of Eq. 14).  First the undeformed
@@ -514,16 +543,10 @@ DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *t
         G = cmul(G, cpow_inv(iU, iU, -ex.eU0));
     }
     /* prod_j (t_j q_j)^{A_j}, t_j only for A_j >= 0: a product with q_j is two FMAs, and 1/q_j = (1 + i d_j)/(1 + d_j^2).
-       The moduli 1 + d_j^2 share one reciprocal while their product is moderate.  d_j carries the scale of the kinematics
-       (F~ is not normalised), so before lambda has been halved far enough it can be anything: then the factors are
-       divided out one by one. */
+       The moduli 1 + d_j^2 share one reciprocal while their product stays below 2^200. */
     double re = s.D, den = 1.0;
-    if (s.sigma > 0) {
-#pragma unroll
-        for (int j = 0; j < S; ++j)
-            for (int k = 0; k > s.A[j]; --k) den *= fma(d[j], d[j], 1.0);
-    }
-    const bool shared_den = biased_exp(den) < 1023u + QMC_SHARED_DEN_EXP; /* den >= 1; false for infinities and NaN */
+    const cd G1 = G;
+    int size = 0;
 #pragma unroll
     for (int j = 0; j < S; ++j) {
         for (int k = 0; k < s.A[j]; ++k) {
@@ -531,30 +554,30 @@ DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *t
             G = mk(fma(G.y, d[j], G.x), fma(-G.x, d[j], G.y));
         }
         for (int k = 0; k > s.A[j]; --k) {
-            if (shared_den) {
-                G = mk(fma(-G.y, d[j], G.x), fma(G.x, d[j], G.y));
-            } else {
-                const double f = __drcp_rn(fma(d[j], d[j], 1.0));
-                G = cmul(G, mk(f, d[j] * f));
-            }
+            den *= fma(d[j], d[j], 1.0);
+            G = mk(fma(-G.y, d[j], G.x), fma(G.x, d[j], G.y));
+            size += modulus_exponent(d[j]);
         }
     }
-    if (s.sigma > 0 && shared_den) re *= qrcp(den);
+    if (size > 200) {
+        Contour<S> c;
+#pragma unroll
+        for (int j = 0; j < S; ++j) c.d[j] = d[j];
+        G = times_q<S>(s, c, G1);
+        den = 1.0;
+    }
+    if (s.sigma > 0) re *= qrcp(den);
     G0 = cscale(G, re);
     X = mk(0.0, 0.0);
     if (needX) {
         /* eU1 log U - eF1 log F + sum_j B_j log q_j (and B_j log t_j where A_j != -1).  The moduli of U and of the q_j
-           share one logarithm, of num / dnm.  Both are products of up to |eU1| + sum |B_j| factors that grow with the
-           kinematics (U through z), so their exponents are added up first (integers, off the FP64 pipe); where they
-           could leave the normal range the mantissas are multiplied and the exponents join as a multiple of ln 2.
-           Without and with the
-           check, 16 shifts: non-planar double box n = 16381 34.26, 34.34 ms; massive box n = 262139 4.79, 4.76 ms. */
+           share one logarithm while their product stays within 2^-1000 to 2^1000. */
         const double U2 = fma(U.x, U.x, U.y * U.y);
         double num = 1.0, dnm = 1.0, xr = 0.0;
         double xi = (double)ex.eU1 * qatan2(U.y, U.x);
         for (int k = 0; k < ex.eU1; ++k) num *= U2;
         for (int k = 0; k > ex.eU1; --k) dnm *= U2;
-        int range = abs(ex.eU1) * exp_size(U2);
+        size = abs(ex.eU1) * (abs(exponent(U2)) + 1);
 #pragma unroll
         for (int j = 0; j < S; ++j) {
             if (s.B[j] != 0) {
@@ -562,20 +585,20 @@ DEV void eval_G(const PackedSector &s, const Pol &P, unsigned Y, const double *t
                 const double q2 = fma(d[j], d[j], 1.0);
                 for (int k = 0; k < s.B[j]; ++k) num *= q2;
                 for (int k = 0; k > s.B[j]; --k) dnm *= q2;
-                range += abs(s.B[j]) * exp_size(q2);
+                size += abs(s.B[j]) * modulus_exponent(d[j]);
                 xi = fma(-qmc_sec.B[j], qatan2(d[j], 1.0), xi);
             }
         }
-        int e2 = 0;
-        if (range > 1000) {
-            num = dnm = 1.0;
-            mul_mantissa(num, dnm, e2, U2, ex.eU1);
-#pragma unroll
-            for (int j = 0; j < S; ++j) mul_mantissa(num, dnm, e2, fma(d[j], d[j], 1.0), s.B[j]);
-        }
         const double eF1 = (double)ex.eF1;
-        double l = qlog(num * qrcp(dnm));
-        if (e2 != 0) l = fma((double)e2, 0.6931471805599453, l);
+        double l;
+        if (size > 1000) {
+            Contour<S> c;
+#pragma unroll
+            for (int j = 0; j < S; ++j) c.d[j] = d[j];
+            l = log_moduli<S>(s, c, U2, ex.eU1);
+        } else {
+            l = qlog(num * qrcp(dnm));
+        }
         X.x = fma(0.5, fma(-eF1, qlog(F2), l), xr);
         X.y = fma(-eF1, arg_mi0(F), xi);
     }

@@ -24,6 +24,8 @@ SHIM = r"""
 #include <cstdlib>
 #include "qmc_internal.h"
 using std::abs;
+#define __device__
+#define __noinline__ static
 struct cd { double x, y; };
 DEV cd mk(double x, double y) { return cd{x, y}; }
 DEV cd csub(cd a, cd b) { return cd{a.x - b.x, a.y - b.y}; }
